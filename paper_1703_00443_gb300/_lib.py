@@ -29,7 +29,7 @@ def _variants():
     for T, tag, pairs in (("float", "f32", [(1, 1), (2, 1), (4, 1), (4, 2)]),
                           ("double", "f64", [(1, 1), (2, 1)])):
         out.append((f"fwd_{tag}_large", "qp_fwd_variant", [f"-DQP_T={T}", "-DQP_KIND=1"]))
-        for kind, kname in ((0, "plain"), (2, "pksmem"), (3, "pkboth")):
+        for kind, kname in ((0, "plain"), (2, "packed")):
             for sw, ch in pairs:
                 out.append((f"fwd_{tag}_{kname}_{sw}{ch}", "qp_fwd_variant",
                             [f"-DQP_T={T}", f"-DQP_KIND={kind}", f"-DQP_SW={sw}", f"-DQP_CH={ch}"]))

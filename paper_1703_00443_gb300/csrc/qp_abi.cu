@@ -66,6 +66,19 @@ size_t fwd_smem(int dtype, int n, int nz, int nineq, int neq, bool large) {
   return L.total;
 }
 
+// Whether the global-memory path's Cholesky panels are in shared memory (then several blocks may
+// share an instance: the panels' place in the workspace is their exchange buffer).
+bool panels_in_smem(int dtype, int n, int nz, int nineq, int neq) {
+  if (dtype == QP_F32) {
+    qpk::FwdSmem<float> L;
+    L.init(n, nz, nineq, neq, true);
+    return L.pan_smem != 0;
+  }
+  qpk::FwdSmem<double> L;
+  L.init(n, nz, nineq, neq, true);
+  return L.pan_smem != 0;
+}
+
 size_t bwd_smem(int dtype, int n, int nz, int nineq, int neq, bool staged = false) {
   if (dtype == QP_F32) {
     qpk::BwdSmem<float> L;
@@ -82,6 +95,8 @@ size_t bwd_smem(int dtype, int n, int nz, int nineq, int neq, bool staged = fals
 // sizes and the device's shared-memory limit, so forward and backward always agree.
 struct Plan {
   bool ok = false, large = false, bstaged = false;
+  bool wide = false;    // global-memory path: products that several blocks may share
+  bool share = false;   // and there is room for them to
   int sw = 0, ch = 0, nz = 0;
   size_t fsmem = 0, bsmem = 0, bsmem_staged = 0, ws = 0;
 };
@@ -107,6 +122,8 @@ Plan make_plan(int dtype, int n, int nineq, int neq, int force_global = 0, bool 
     pl.nz = n + ((qpk::LNB - (n + neq) % qpk::LNB) % qpk::LNB);
   }
   pl.fsmem = fwd_smem(dtype, n, pl.nz, nineq, neq, pl.large);
+  pl.wide = pl.large && qpk::wide_size(pl.nz + neq);
+  pl.share = pl.wide && panels_in_smem(dtype, n, pl.nz, nineq, neq);
   pl.bsmem = bwd_smem(dtype, n, pl.nz, nineq, neq);
   // The fixed-size backward kernel stages S/RE and X in shared memory when they fit there.
   if (!pl.large) {
@@ -127,15 +144,15 @@ Plan make_plan(int dtype, int n, int nineq, int neq, int force_global = 0, bool 
 
 static_assert(sizeof(qp_instance_desc) == sizeof(qpk::PackedDesc), "descriptor layout");
 
-// Non-blocking side streams, each with a fork/join event pair, created on first use (host-side
+// Non-blocking side streams with their fork/join events, created on first use (host-side
 // resources, not device memory) and kept for the life of the process.  A caller's stream
-// gets its own side stream (up to kSideSlots per device; beyond that, streams share slots by
+// gets its own set (up to kSideSlots per device; beyond that, streams share sets by
 // hash), so packed calls issued on different streams do not queue behind one another.
 struct SideStream {
   cudaStream_t owner = nullptr;   // the caller stream this slot serves
   bool used = false;
-  cudaStream_t s = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaStream_t s[3] = {nullptr, nullptr, nullptr};
+  cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
   std::mutex mu;
 };
 constexpr int kSideSlots = 16;
@@ -157,9 +174,13 @@ SideStream* side_stream(cudaStream_t owner) {
     if (!row[i].used) x = &row[i];
   if (!x) x = &row[(reinterpret_cast<uintptr_t>(owner) >> 4) % kSideSlots];
   if (!x->used) {
-    if (cudaStreamCreateWithFlags(&x->s, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&x->join, cudaEventDisableTiming) != cudaSuccess) {
+    bool ok = x->fork || cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < 3; ++i) {
+      ok = ok && (x->s[i] || cudaStreamCreateWithFlags(&x->s[i], cudaStreamNonBlocking) == cudaSuccess);
+      ok = ok && (x->join[i] ||
+                  cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess);
+    }
+    if (!ok) {
       cudaGetLastError();
       return nullptr;
     }
@@ -185,6 +206,26 @@ double est_cost(int n, int nz, int p, int m, bool large) {
   const double m1 = nz + m, N = m1 + p;
   const double c = m1 * N * N + 12.0 * (p * (double)p * p / 3.0 + 2.0 * n * N) + N * N;
   return large ? 3.0 * c : c;
+}
+
+// Blocks per instance on the global-memory path for a batch of B: a cluster of up to eight while
+// the whole batch's clusters are resident at once (one block per SM; a cluster needs its SMs
+// within one processing cluster of 16 to 20, which leaves a few SMs unused), one block otherwise.
+#if defined(QP_HOST_EMULATION)
+constexpr int kQueuedBlocks = 1;
+#else
+constexpr int kQueuedBlocks = 4;
+#endif
+int blocks_per_instance(int B, bool share) {
+#if defined(QP_HOST_EMULATION)
+  return 1;   // the host emulation runs one block at a time
+#endif
+  const int nsm = num_sms();
+  if (!share) return 1;
+  if (B * 8 <= nsm * 3 / 4) return 8;
+  if (B * 4 <= nsm * 9 / 10) return 4;
+  if (B * 2 <= nsm * 9 / 10) return 2;
+  return 1;
 }
 
 namespace qpk {
@@ -258,13 +299,14 @@ int qp_forward(const qp_options* opt, int dtype, int B, int n, int nineq, int ne
   if (workspace_bytes < (size_t)B * pl.ws) return QP_ENOSPACE;
   if (!pl.ok) return QP_EUNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
+  const int blocks = pl.wide ? blocks_per_instance(B, pl.share) : 0;
   cudaError_t e;
   if (dtype == QP_F32) {
     qpk::FwdParams<float> P{B, n, nineq, neq, pl.nz,
                             (const float*)Q, (const float*)q, (const float*)G, (const float*)h,
                             (const float*)A, (const float*)b, (float*)z, (float*)lam, (float*)nu,
                             status, iters, resid, (unsigned char*)workspace,
-                            pl.ws, o.tol, o.mu_tol, o.max_iter, tl_ns};
+                            pl.ws, o.tol, o.mu_tol, o.max_iter, tl_ns, blocks};
     e = pl.large ? qpk::launch_fwd_large_f32(P, pl.fsmem, st)
                  : qpk::launch_fwd_f32(P, pl.sw, pl.ch, pl.fsmem, st);
   } else {
@@ -272,7 +314,7 @@ int qp_forward(const qp_options* opt, int dtype, int B, int n, int nineq, int ne
                              (const double*)Q, (const double*)q, (const double*)G, (const double*)h,
                              (const double*)A, (const double*)b, (double*)z, (double*)lam,
                              (double*)nu, status, iters, resid, (unsigned char*)workspace,
-                             pl.ws, o.tol, o.mu_tol, o.max_iter, tl_ns};
+                             pl.ws, o.tol, o.mu_tol, o.max_iter, tl_ns, blocks};
     e = pl.large ? qpk::launch_fwd_large_f64(P, pl.fsmem, st)
                  : qpk::launch_fwd_f64(P, pl.sw, pl.ch, pl.fsmem, st);
   }
@@ -346,6 +388,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   int64_t ows = 256;   // first 256 bytes: the two work-queue counters
   int sw_need = 1, ch_need = 1;
   size_t fsm = 0, bsm = 0;
+  int nwide = 0, nshare = 0;
   std::vector<std::pair<double, int>> order;
   for (int i = 0; i < B; ++i) {
     const int n = dims[3 * i], p = dims[3 * i + 1], m = dims[3 * i + 2];
@@ -355,7 +398,8 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     const Plan pl = make_plan(dtype, n, p, m, hint ? hint : o.path, true);
     if (!pl.ok) return QP_EUNSUPPORTED;
     qp_instance_desc& d = desc[i];
-    d.n = n; d.nineq = p; d.neq = m; d.id = i; d.nz = pl.nz; d.flags = pl.large ? 1 : 0;
+    d.n = n; d.nineq = p; d.neq = m; d.id = i; d.nz = pl.nz;
+    d.flags = (pl.large ? 1 : 0) | (pl.wide ? 2 : 0);
     d.oQ = oQ; d.oq = oq; d.oG = oG; d.oh = oh; d.oA = oA; d.ob = ob;
     d.oz = oq; d.olam = oh; d.onu = ob; d.ows = ows;
     // Offsets padded to multiples of 4 elements keep every instance's rows 16-byte aligned.
@@ -368,6 +412,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
       ch_need = std::max(ch_need, pl.ch);
     } else {
       ++S.n_global;
+      if (pl.wide) ++nwide;
     }
     fsm = std::max(fsm, pl.fsmem);
     bsm = std::max(bsm, pl.bsmem);
@@ -380,12 +425,13 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     for (int k = 0; k < 3; ++k)
       if (sws[k] >= sw_need && qpk::fwd_variant_exists(esz, sws[k], c)) { sw = sws[k]; ch = c; break; }
   if (!sw) return QP_EUNSUPPORTED;
-  // Execution order: global-path instances first, then shared-memory-path ones (the two run
-  // as separate kernels), each part largest estimated cost first (longest-processing-time).
+  // Execution order: the global-path instances of wide sizes first, then the other global-path
+  // ones, then the shared-memory-path ones (separate kernels), each part largest estimated cost
+  // first (longest-processing-time).
   std::vector<qp_instance_desc> tmp(desc, desc + B);
   std::stable_sort(order.begin(), order.end(),
                    [&](const std::pair<double, int>& x, const std::pair<double, int>& y) {
-                     const int gx = tmp[x.second].flags & 1, gy = tmp[y.second].flags & 1;
+                     const int gx = tmp[x.second].flags & 3, gy = tmp[y.second].flags & 3;
                      return gx != gy ? gx > gy : x.first > y.first;
                    });
   for (int k = 0; k < B; ++k) desc[k] = tmp[order[k].second];
@@ -394,6 +440,18 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   S.ws_bytes = ows;
   S.fwd_smem = (int64_t)fsm; S.bwd_smem = (int64_t)bsm;
   S.sw = sw; S.ch = ch;
+  // Wide instances to share among several blocks: the leading ones (largest first) whose own
+  // estimated time on one SM would exceed 1.2 of the batch's total over all SMs, and so set
+  // the batch's time.  The plan keeps both counts in `reserved`.
+  double total = 0.0;
+  for (const auto& x : order) total += x.first;
+  const double limit = 1.2 * total / num_sms();
+  while (nshare < std::min(nwide, 255) && order[nshare].first > limit) {
+    const qp_instance_desc& d = desc[nshare];
+    if (!panels_in_smem(dtype, d.n, d.nz, d.nineq, d.neq)) break;
+    ++nshare;
+  }
+  S.reserved = nwide << 8 | nshare;
   *sizes = S;
   return QP_OK;
 }
@@ -415,55 +473,70 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
   if (o.max_iter < 0 || o.time_limit_us < 0) return QP_EINVAL;
   const unsigned long long tl_ns = 1000ull * (unsigned long long)o.time_limit_us;
   cudaStream_t st = (cudaStream_t)stream;
-  // Work-queue counters: bytes 0..3 the shared-memory-path kernel's, 4..7 the backward's,
-  // 8..11 the kernel of the global-path instances.
+  // Work-queue counters: bytes 0..3 the shared-memory-path kernel's, 4..7 the backward's.
   if (cudaMemsetAsync(workspace, 0, 16, st) != cudaSuccess) return QP_ECUDA;
   const int nsm = num_sms(), ng = std::min(std::max(sizes->n_global, 0), B), ns = B - ng;
-  auto launch = [&](int mode, int off, int cnt, int grid, int ctr_byte, cudaStream_t s) {
+  // kind −1: shared-memory-path instances [off, off + cnt); 0: global-path ones of sizes that are
+  // not wide; otherwise wide ones with `kind` blocks each.
+  auto launch = [&](int kind, int off, int cnt, cudaStream_t s) {
+    const int grid = std::min(cnt, nsm);
     if (dtype == QP_F32) {
-      qpk::PackedFwdParams<float> P{cnt, (const qpk::PackedDesc*)desc + off,
-                                    (int*)((char*)workspace + ctr_byte),
+      qpk::PackedFwdParams<float> P{cnt, (const qpk::PackedDesc*)desc + off, (int*)workspace,
                                     (const float*)Q, (const float*)q, (const float*)G,
                                     (const float*)h, (const float*)A, (const float*)b, (float*)z,
                                     (float*)lam, (float*)nu, status, iters, resid,
-                                    (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns};
-      return qpk::launch_fwd_packed_f32(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem, grid,
-                                        mode, s);
+                                    (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns,
+                                    kind};
+      return kind >= 0 ? qpk::launch_fwd_packed_large_f32(P, (size_t)sizes->fwd_smem, s)
+                  : qpk::launch_fwd_packed_f32(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem,
+                                               grid, s);
     }
-    qpk::PackedFwdParams<double> P{cnt, (const qpk::PackedDesc*)desc + off,
-                                   (int*)((char*)workspace + ctr_byte),
+    qpk::PackedFwdParams<double> P{cnt, (const qpk::PackedDesc*)desc + off, (int*)workspace,
                                    (const double*)Q, (const double*)q, (const double*)G,
                                    (const double*)h, (const double*)A, (const double*)b,
                                    (double*)z, (double*)lam, (double*)nu, status, iters, resid,
-                                   (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns};
-    return qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem, grid,
-                                      mode, s);
+                                   (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns,
+                                   kind};
+    return kind >= 0 ? qpk::launch_fwd_packed_large_f64(P, (size_t)sizes->fwd_smem, s)
+                : qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem,
+                                             grid, s);
   };
-  cudaError_t e;
-  if (ns == 0) {
-    e = launch(qpk::PK_BOTH, 0, ng, std::min(ng, nsm), 8, st);
-  } else if (ng == 0) {
-    e = launch(qpk::PK_SMEM, 0, ns, std::min(ns, nsm), 0, st);
-  } else {
-    // Both kinds: the global-path instances (first in the descriptor array) in the combined
-    // kernel on `stream`, launched first so that its blocks take the SMs first; the
-    // shared-memory-path instances in the shared-memory-only kernel on a side stream forked
-    // from `stream` and joined back to it.  Each block of either kernel holds its SM until its
-    // queue runs dry, so as global-path blocks finish, shared-memory-path blocks take their
-    // SMs: the hardware block scheduler balances the two queues without a fixed split.
-    SideStream* ss = side_stream(st);
-    if (!ss) return QP_ECUDA;
-    std::lock_guard<std::mutex> lk(ss->mu);
-    if (cudaEventRecord(ss->fork, st) != cudaSuccess) return QP_ECUDA;
-    e = launch(qpk::PK_BOTH, 0, ng, std::min(ng, nsm), 8, st);
-    if (e != cudaSuccess) return QP_ECUDA;
-    if (cudaStreamWaitEvent(ss->s, ss->fork, 0) != cudaSuccess) return QP_ECUDA;
-    e = launch(qpk::PK_SMEM, ng, ns, std::min(ns, nsm), 0, ss->s);
-    if (cudaEventRecord(ss->join, ss->s) != cudaSuccess ||
-        cudaStreamWaitEvent(st, ss->join, 0) != cudaSuccess)
+  // Up to four kernels side by side: the largest wide instances with several blocks each (first
+  // in the descriptor array), the other wide ones, the other global-path ones, and the
+  // shared-memory-path ones; the first of them on `stream`, the others on side streams forked
+  // from it and joined back to it, launched in this order so that the costliest take the SMs
+  // first.  A block holds its SM until it ends (the last kernel's until its queue runs dry), so
+  // as blocks finish, the next kernel's take their SMs: the hardware block scheduler
+  // balances the queues without a fixed split.
+  struct Part { int kind, off, cnt; } parts[4];
+  int np = 0;
+  const int nwide = std::min(std::max(sizes->reserved >> 8, 0), ng);
+  const int nshare = std::min(sizes->reserved & 255, nwide);
+  // (four blocks each where the clusters take turns)
+  if (nshare > 0) parts[np++] = {std::max(blocks_per_instance(nshare, true), kQueuedBlocks), 0, nshare};
+  if (nwide > nshare) parts[np++] = {1, nshare, nwide - nshare};
+  if (ng > nwide) parts[np++] = {0, nwide, ng - nwide};
+  if (ns > 0) parts[np++] = {-1, ng, ns};
+  if (np == 1) {
+    const cudaError_t e = launch(parts[0].kind, parts[0].off, parts[0].cnt, st);
+    return e == cudaSuccess ? QP_OK : QP_ECUDA;
+  }
+  SideStream* ss = side_stream(st);
+  if (!ss) return QP_ECUDA;
+  std::lock_guard<std::mutex> lk(ss->mu);
+  if (cudaEventRecord(ss->fork, st) != cudaSuccess) return QP_ECUDA;
+  if (launch(parts[0].kind, parts[0].off, parts[0].cnt, st) != cudaSuccess) return QP_ECUDA;
+  bool ok = true;
+  for (int i = 1; i < np; ++i) {
+    cudaStream_t s = ss->s[i - 1];
+    if (cudaStreamWaitEvent(s, ss->fork, 0) != cudaSuccess) return QP_ECUDA;
+    ok = launch(parts[i].kind, parts[i].off, parts[i].cnt, s) == cudaSuccess && ok;
+    // joined whether or not the launch succeeded
+    if (cudaEventRecord(ss->join[i - 1], s) != cudaSuccess ||
+        cudaStreamWaitEvent(st, ss->join[i - 1], 0) != cudaSuccess)
       return QP_ECUDA;
   }
-  return e == cudaSuccess ? QP_OK : QP_ECUDA;
+  return ok ? QP_OK : QP_ECUDA;
 }
 
 int qp_backward_packed(const qp_options* opt, int dtype, int B, const qp_instance_desc* desc,

@@ -42,8 +42,9 @@ constexpr int NWARPS = NTHREADS / 32;
 // the staged inverse diagonal block (32 × 33).
 constexpr int BLK_SOLVE_SCR = 32 + 32 * NWARPS + 32 * 33;
 // Shared-memory budget (bytes) under which the global-memory path keeps its Cholesky panels
-// in shared memory; below every supported device's opt-in limit of the target (227 KB).
-constexpr size_t LARGE_PANEL_SMEM_CAP = 200 * 1024;
+// in shared memory: the opt-in limit of the target (227 KB) less room for static shared memory.
+// (At 200 KB the panels of p = 500 went to global memory.)
+constexpr size_t LARGE_PANEL_SMEM_CAP = 226 * 1024;
 // Column block of the global-memory Cholesky: 32 for FP32, 16 for FP64 (one warp holds the
 // pivot block's row and its inverse's row in registers).
 __host__ __device__ constexpr int chol_nb(int esz) { return esz == 4 ? 32 : 16; }
@@ -202,7 +203,7 @@ struct FwdSmem {
       // The setup sweep's two 16-row panels (ld round8(m1 + p)) likewise, after its pivot
       // scratch, if they fit too.
       const size_t nb = (size_t)chol_nb((int)es);
-      const size_t pc = align_up(((2 * nb * nb + 2 * nb + 16) + 2 * nb * (size_t)((p + 7) & ~7)) * es, 16);
+      const size_t pc = align_up(((2 * nb * nb + 10 * nb + 16) + 2 * nb * (size_t)((p + 7) & ~7)) * es, 16);
       const size_t sc = align_up((2 * 16 * 16 + 16 + 2 * 16 * (size_t)((N3 + 7) & ~7)) * es, 16);
       if (o + (pc > cbytes ? pc : cbytes) + tail <= LARGE_PANEL_SMEM_CAP) {
         pan_smem = 1;
@@ -261,6 +262,7 @@ struct FwdParams {
   double tol, mu_tol;
   int max_iter;
   unsigned long long time_limit_ns;   // 0: none
+  int blocks;   // global-memory path: blocks per instance of a wide size, 0 for the others
 };
 
 // Per-instance views used by the kernel bodies (built from the fixed-size parameters or from
@@ -309,6 +311,7 @@ struct PackedFwdParams {
   double tol, mu_tol;
   int max_iter;
   unsigned long long time_limit_ns;
+  int blocks;   // global-memory-path launches: as in FwdParams
 };
 
 template <typename T>
@@ -942,6 +945,289 @@ __device__ __forceinline__ void kkt_apply_fast(int n, int p, int m, const T* __r
   __syncthreads();
 }
 
+// ------------------------------------------------------------------ products over a cluster
+// The global-memory path may run an instance on a cluster of several blocks: each block keeps
+// the vectors and takes every scalar decision itself, on identical values, and the blocks
+// split the work on the matrices.  A product's rows (or columns) are dealt to the warps of
+// all blocks and the results exchanged through `ex`, a buffer in the instance's workspace;
+// the summation order depends on the sizes alone, so results do not depend on the number of
+// blocks.  With one block the results go straight to shared memory.
+template <typename T>
+struct Dist {
+  int blocks, rank;
+  T* ex;          // exchange buffer (workspace)
+  int cap;        // its size in elements of T
+};
+
+// Sizes that take these products: below them one block's registers and its own shared-memory
+// partial sums are faster (n = 200, nineq = 150: 2.6 ms a batch of 128 against 4.3).
+__host__ __device__ inline bool wide_size(int m1) { return m1 >= 352; }
+
+// out[r] = Σ_c M[r·ld + c]·x[c] over all c < cols (upper = false) or c > r, eight lanes per row,
+// for the rows dealt to this block.  x is shared memory.  No barrier inside.  Loads go in
+// batches of eight per lane with the tail masked: a remainder loop would wait for L2 one load
+// after the other.
+template <typename T>
+__device__ __noinline__ void dist_rows(const Dist<T>& D, const T* M, int ld, int rows, int cols,
+                                          bool upper, const T* x, T* out) {
+  constexpr int GL = 8, NG = NTHREADS / GL, W = 16 / sizeof(T);
+  const int g = threadIdx.x / GL, gl = threadIdx.x % GL;
+  const bool vec = !upper && ld % W == 0 && cols % W == 0;
+#pragma unroll 1
+  for (int r0 = D.rank * NG; r0 < rows; r0 += D.blocks * NG) {
+    const int r = r0 + g;
+    const T* row = M + (size_t)r * ld;
+    T a0 = T(0), a1 = T(0);
+    if (r < rows) {
+      if (vec) {
+        constexpr int U = 8;
+#pragma unroll 1
+        for (int cb = W * gl; cb < cols; cb += GL * W * U) {
+          T a[U][W];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int c = cb + GL * W * u;
+            if constexpr (W == 4) {
+              const float4 t = c < cols ? *reinterpret_cast<const float4*>(row + c)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+              a[u][0] = t.x; a[u][1] = t.y; a[u][2] = t.z; a[u][3] = t.w;
+            } else {
+              const double2 t = c < cols ? *reinterpret_cast<const double2*>(row + c)
+                                         : make_double2(0.0, 0.0);
+              a[u][0] = t.x; a[u][1] = t.y;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int c = cb + GL * W * u;
+            if (c < cols) {
+#pragma unroll
+              for (int e = 0; e < W; ++e) {
+                if (e & 1) a1 = fma(a[u][e], x[c + e], a1);
+                else a0 = fma(a[u][e], x[c + e], a0);
+              }
+            }
+          }
+        }
+      } else {
+        constexpr int U = 16;
+#pragma unroll 1
+        for (int cb = (upper ? r + 1 : 0) + gl; cb < cols; cb += GL * U) {
+          T a[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) a[u] = cb + GL * u < cols ? row[cb + GL * u] : T(0);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (cb + GL * u < cols) a0 = fma(a[u], x[cb + GL * u], a0);
+        }
+      }
+    }
+    T s = a0 + a1;
+#pragma unroll
+    for (int off = GL / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (r < rows && gl == 0) out[r] = s;
+  }
+}
+
+// A column product's items: 32 columns (FP32 rows on vector boundaries: 128, four per lane, which
+// keeps twice the bytes in flight) and a row range, enough of them for 128 warps.
+template <typename T>
+__device__ __forceinline__ int dist_col_width(int ld, int cols) {
+  return sizeof(T) == 4 && ld % 4 == 0 && cols % 4 == 0 ? 128 : 32;
+}
+template <typename T>
+__device__ __forceinline__ int dist_col_parts(int ld, int rows, int cols) {
+  const int w = dist_col_width<T>(ld, cols);
+  return max(1, min(min(16, 128 / ((cols + w - 1) / w)), (rows + 3) >> 2));
+}
+
+// Partial sums out[part·cols + c] of Σ_r M[r·ld + c]·x[r] over all r < rows (upper = false) or
+// r < c, one warp per item, for the items dealt to this block.
+template <typename T>
+__device__ __noinline__ void dist_cols(const Dist<T>& D, const T* M, int ld, int rows, int cols,
+                                       bool upper, const T* x, T* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int w = dist_col_width<T>(ld, cols), ng = (cols + w - 1) / w;
+  const int nparts = dist_col_parts<T>(ld, rows, cols);
+#pragma unroll 1
+  for (int e = D.rank * NWARPS + warp; e < ng * nparts; e += D.blocks * NWARPS) {
+    const int part = e / ng, g = e - part * ng;
+    const int rmax = upper ? min(rows, w * g + w) : rows;
+    const int chunk = (rmax + nparts - 1) / nparts;
+    const int r0 = part * chunk, rend = min(rmax, r0 + chunk);
+    if constexpr (sizeof(T) == 4) {
+      if (w == 128) {
+        const int c = 128 * g + 4 * lane;
+        if (c >= cols) continue;
+        const int r1 = upper ? min(rend, c + 3) : rend;   // rows < some column of the four
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int r = r0; r < r1; r += 8) {
+          float4 v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            v[u] = r + u < r1 ? *reinterpret_cast<const float4*>(M + (size_t)(r + u) * ld + c)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (r + u < r1) {
+              const float t = x[r + u];
+              // (upper: entries on and below the diagonal belong to the factor)
+              if (!upper || r + u < c) a[0] = fmaf(v[u].x, t, a[0]);
+              if (!upper || r + u < c + 1) a[1] = fmaf(v[u].y, t, a[1]);
+              if (!upper || r + u < c + 2) a[2] = fmaf(v[u].z, t, a[2]);
+              if (!upper || r + u < c + 3) a[3] = fmaf(v[u].w, t, a[3]);
+            }
+        }
+        *reinterpret_cast<float4*>(out + part * cols + c) = make_float4(a[0], a[1], a[2], a[3]);
+        continue;
+      }
+    }
+    const int c = 32 * g + lane;
+    if (c >= cols) continue;
+    const int r1 = upper ? min(rend, c) : rend;
+    T a0 = T(0), a1 = T(0);
+#pragma unroll 1
+    for (int r = r0; r < r1; r += 16) {
+      T a[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) a[u] = r + u < r1 ? M[(size_t)(r + u) * ld + c] : T(0);
+#pragma unroll
+      for (int u = 0; u < 16; u += 2) {
+        if (r + u < r1) a0 = fma(a[u], x[r + u], a0);
+        if (r + u + 1 < r1) a1 = fma(a[u + 1], x[r + u + 1], a1);
+      }
+    }
+    out[part * cols + c] = a0 + a1;
+  }
+}
+template <typename T>
+__device__ __forceinline__ T dist_col_sum(const T* parts, int cols, int nparts, int c) {
+  // the parts are at most 16: their loads in flight together
+  T a = T(0);
+#pragma unroll
+  for (int q0 = 0; q0 < 16; q0 += 8) {
+    T v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = q0 + e < nparts ? parts[(q0 + e) * cols + c] : T(0);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) a += v[e];
+  }
+  return a;
+}
+
+// The KKT operator (kkt_apply) over a cluster, added to the outputs: partial column sums of row ranges and the row
+// products go through the exchange buffer as accumulators.
+// Row ranges of the column pass (about 32 rows) for an exchange buffer of `bytes` bytes after the row results.
+__device__ __forceinline__ int dist_kkt_parts(int n, int R, size_t bytes) {
+  const int nq = (n + 3) >> 2;
+  return max(1, min((R + 31) >> 5, (int)(bytes / (8 * 4 * (size_t)nq))));
+}
+template <typename T>
+__device__ __noinline__ void dist_kkt(const Dist<T>& D, int n, int p, int m,
+                                         const T* __restrict__ Q, const T* __restrict__ G,
+                                         const T* __restrict__ A, const typename Split<T>::V* xv,
+                                         double* out_z, double* out_l, double* out_n) {
+  using V = typename Split<T>::V;
+  using AC = Acc<T>;
+  const int tid = threadIdx.x, R = n + p + m, nq = (n + 3) >> 2;
+  const bool vec = (n % 4 == 0) &&
+      ((((uintptr_t)Q) | ((uintptr_t)G) | ((uintptr_t)A)) % (4 * sizeof(T)) == 0);
+  auto rowp = [&](int r) -> const T* {
+    return r < n ? Q + (size_t)r * n : (r < n + p ? G + (size_t)(r - n) * n : A + (size_t)(r - n - p) * n);
+  };
+  AC* rowres = reinterpret_cast<AC*>(D.ex);
+  const size_t rb = 8 * (size_t)((p + m + 1) & ~1);
+  AC* parts = reinterpret_cast<AC*>(reinterpret_cast<unsigned char*>(D.ex) + rb);
+  const int nparts = dist_kkt_parts(n, R, (size_t)D.cap * sizeof(T) - rb);
+  const int chunk = (R + nparts - 1) / nparts;
+  // column pass: quads of columns over row ranges
+  for (int t = D.rank * NTHREADS + tid; t < nq * nparts; t += D.blocks * NTHREADS) {
+    const int part = t / nq, jq = t - part * nq;
+    const int r0 = part * chunk, r1 = min(R, r0 + chunk);
+    constexpr int RB = sizeof(T) == 4 ? 8 : 4;
+    AC acc[4];
+#pragma unroll 1
+    for (int r = r0; r < r1; r += RB) {
+      T av[RB][4];
+#pragma unroll
+      for (int u = 0; u < RB; ++u)
+        if (r + u < r1) ldg4_row(av[u], rowp(r + u), 4 * jq, n, vec);
+#pragma unroll
+      for (int u = 0; u < RB; ++u)
+        if (r + u < r1) {
+          const V x = xv[r + u];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c].add(av[u][c], x);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) parts[(size_t)part * 4 * nq + 4 * jq + c] = acc[c];
+  }
+  // row pass: eight lanes per row, two rows per lane group
+  {
+    constexpr int GL = 8, NG = NTHREADS / GL, QB = 4;
+    const int g = tid / GL, gl = tid % GL;
+    for (int r0 = D.rank * 2 * NG; r0 < p + m; r0 += D.blocks * 2 * NG) {
+      const int rr[2] = {r0 + g, r0 + NG + g};
+      const T* rowv[2];
+#pragma unroll
+      for (int h2 = 0; h2 < 2; ++h2) rowv[h2] = rowp(n + min(rr[h2], p + m - 1));
+      AC acc[2];
+      for (int qb0 = 0; qb0 < nq; qb0 += GL * QB) {
+        T av[2][QB][4];
+#pragma unroll
+        for (int h2 = 0; h2 < 2; ++h2)
+#pragma unroll
+          for (int u = 0; u < QB; ++u) {
+            const int q = qb0 + gl + u * GL;
+            if (q < nq) ldg4_row(av[h2][u], rowv[h2], 4 * q, n, vec);
+          }
+#pragma unroll
+        for (int u = 0; u < QB; ++u) {
+          const int q = qb0 + gl + u * GL;
+          if (q < nq) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              if (4 * q + c < n) {
+                const V x = xv[4 * q + c];
+                acc[0].add(av[0][u][c], x);
+                acc[1].add(av[1][u][c], x);
+              }
+          }
+        }
+      }
+#pragma unroll
+      for (int h2 = 0; h2 < 2; ++h2) {
+#pragma unroll
+        for (int off = GL / 2; off > 0; off >>= 1) acc[h2].shfl_merge(off);
+        if (rr[h2] < p + m && gl == 0) rowres[rr[h2]] = acc[h2];
+      }
+    }
+  }
+  cluster_barrier(D.blocks);
+  for (int j = tid; j < n; j += NTHREADS) {
+    AC acc;
+#pragma unroll 1
+    for (int q0 = 0; q0 < nparts; q0 += 8) {
+      AC v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (q0 + e < nparts) v[e] = parts[(size_t)(q0 + e) * 4 * nq + j];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (q0 + e < nparts) acc.merge(v[e]);
+    }
+    out_z[j] = acc.value() + out_z[j];
+  }
+  for (int i = tid; i < p + m; i += NTHREADS) {
+    const double v = rowres[i].value();
+    if (i < p) out_l[i] = v + out_l[i];
+    else out_n[i - p] = v + out_n[i - p];
+  }
+  cluster_barrier(D.blocks);
+}
+
 // ------------------------------------------------------------------ register tiles
 // Lower-triangular tiling of an N×N symmetric matrix by 4×4 tiles; linear tile t maps to
 // tile row I = ⌊(√(8t+1) − 1)/2⌋ and tile column J = t − I(I+1)/2.
@@ -1493,12 +1779,13 @@ namespace qpk {
 // shared-memory kernel and the global-memory kernel.  SR (= [S; RE], leading dimension
 // ldS = m1), Mb (M strict upper / X lower, leading dimension ldM) and dM point to shared or
 // global memory; setup() fills them (the setup sweep) and factor(dsh) factors
-// M + D(dsh) into X.  With ws_resident the factors already live in the workspace, otherwise
-// they are copied there for the backward pass.
-template <typename T, typename FS, typename FF, typename FV>
+// M + D(dsh) into X.  With ws_resident the factors already live in the workspace, and the
+// products are those of Dist when WIDE (the instance may then be shared by the blocks of a
+// cluster, D); otherwise the factors are copied there for the backward pass.
+template <typename T, bool ws_resident, bool WIDE, typename FS, typename FF, typename FV>
 __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& L,
                                          unsigned char* sm, T* SR, T* Mb, int ldMb, T* dM,
-                                         bool ws_resident, FS setup, FF factor, FV solve) {
+                                         const Dist<T>& D, FS setup, FF factor, FV solve) {
   using V = typename Split<T>::V;
   const int tid = threadIdx.x;
   const int n = P.n, p = P.p, m = P.m;
@@ -1539,6 +1826,48 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
   int32_t* wSt = reinterpret_cast<int32_t*>(wsb + W.oSt);
   const int ldS = m1, ldM = ldMb;
 
+  // Products with the factors: wv = [S; RE]·u; with_m(x, out, re): out = M·x (M symmetric, strict
+  // upper triangle plus diag) and, when re, dzn = wv − REᵀx.
+  auto with_sr = [&]() {
+    if constexpr (WIDE) {
+      T* o = D.blocks > 1 ? D.ex : wv;
+      dist_rows(D, SR, ldS, m1 + p, m1, false, u, o);
+      cluster_barrier(D.blocks);
+      if (D.blocks > 1) {
+        for (int i = tid; i < m1 + p; i += NTHREADS) wv[i] = o[i];
+        cluster_barrier(D.blocks);
+      }
+    } else {
+      if (!mv_rows_xreg<8>(SR, ldS, m1 + p, m1, u, [&](int r, T val) { wv[r] = val; }))
+        mv_rows<8>(SR, ldS, m1 + p, m1, TRI_ALL, u, [&](int r, T val) { wv[r] = val; });
+      __syncthreads();
+    }
+  };
+  auto with_m = [&](const T* x, T* out, bool mul_m, bool mul_re) {
+    if constexpr (WIDE) {
+      // exchange buffer: row products | column parts of M | column parts of RE
+      const int npm = dist_col_parts<T>(ldM, p, p), npr = dist_col_parts<T>(ldS, p, m1);
+      T *rowp = D.ex, *mp = rowp + p4, *rp = mp + (size_t)npm * p4;
+      const T* RE = SR + (size_t)m1 * ldS;
+      if (mul_m) {
+        dist_rows(D, Mb, ldM, p, p, true, x, rowp);
+        dist_cols(D, Mb, ldM, p, p, true, x, mp);
+      }
+      if (mul_re) dist_cols(D, RE, ldS, p, m1, false, x, rp);
+      cluster_barrier(D.blocks);
+      if (mul_m)
+        for (int i = tid; i < p; i += NTHREADS)
+          out[i] = fma(dM[i], x[i], rowp[i]) + dist_col_sum(mp, p, npm, i);
+      if (mul_re)
+        for (int i = tid; i < m1; i += NTHREADS) dzn[i] = wv[i] - dist_col_sum(rp, m1, npr, i);
+      cluster_barrier(D.blocks);
+    } else {
+      if (mul_re)
+        mv_cols(SR + (size_t)m1 * ldS, ldS, p, m1, TRI_ALL, x, tscr,
+                [&](int c, T val) { dzn[c] = wv[c] - val; }, tcap);
+      if (mul_m) mv_sym_upper(p, Mb, ldM, dM, x, tmp, out, tscr, tcap);
+    }
+  };
   int status = ST_CONV, it = 0, extra = 0, flags = 0;
   float last[4] = {0.f, 0.f, 0.f, 0.f};   // residual norms and μ at the returned iterate
   double cert_scale = 1.0;                 // 1/max(‖λ‖∞, ‖ν‖∞) of an infeasibility certificate
@@ -1553,9 +1882,17 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     for (int i = tid; i < n + p + m; i += NTHREADS)
       xs[i] = Split<T>::make(i < n ? 0.0 : (i < n + p ? lam[i - n] : nu[i - n - p]));
     __syncthreads();
-    kkt_apply<T>(n, p, m, P.Q, p ? P.G : nullptr, m ? P.A : nullptr, xs, ascr, kscr,
-                 [&](int) { return 0.0; }, [&](int) { return 0.0; }, [&](int) { return 0.0; },
-                 rz, rl, rn);
+    auto zero = [](int) { return 0.0; };
+    if constexpr (WIDE)
+    {
+      for (int i = tid; i < max(n, p + m); i += NTHREADS) {
+        if (i < n) rz[i] = 0.0;
+        if (i < p + m) rl[i] = 0.0;   // rl, rn are one array
+      }
+      __syncthreads();
+      dist_kkt<T>(D, n, p, m, Qb, Gb, Ab, xs, rz, rl, rn);
+    } else
+      kkt_apply<T>(n, p, m, Qb, Gb, Ab, xs, ascr, kscr, zero, zero, zero, rz, rl, rn);
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (int i = tid; i < p; i += NTHREADS) {
       v[0] -= hd[i] * lam[i];
@@ -1590,7 +1927,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     qmx = v[0];
   }
   bool ok = setup(Qb, Ab, Gb, T(0), (T)((sizeof(T) == 4 ? 1e-5f : 1e-12f) * qmx));
-  __syncthreads();
+  cluster_barrier(D.blocks);
   if (!ok) {
     float v[4] = {qmx, 0.f, 0.f, 0.f};
     for (int i = tid; i < p + m; i += NTHREADS) {
@@ -1603,7 +1940,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     const float scale = fmaxf(fmaxf(v[0], v[1]), 1e-30f);
     delta = (T)((sizeof(T) == 4 ? 1e-4f : 1e-8f) * scale);
     if (isfinite(scale)) ok = setup(Qb, Ab, Gb, delta, T(0));
-    __syncthreads();
+    cluster_barrier(D.blocks);
     if (ok) flags |= FLAG_REGQ;
   }
   if (!ok) status = ST_NOTPD;
@@ -1664,14 +2001,11 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     ok = factor(dsh);
     if (!ok) status = ST_NOTPD;
     if (ok) {
-      if (!mv_rows_xreg<8>(SR, ldS, m1 + p, m1, u, [&](int r, T val) { wv[r] = val; }))
-        mv_rows<8>(SR, ldS, m1 + p, m1, TRI_ALL, u, [&](int r, T val) { wv[r] = val; });
-      __syncthreads();
+      with_sr();
       for (int i = tid; i < p; i += NTHREADS) rhs[i] = wv[m1 + i] - hb[i];
       __syncthreads();
       solve(rhs, y, dl, tscr);
-      mv_cols(SR + (size_t)m1 * ldS, ldS, p, m1, TRI_ALL, dl, tscr,
-              [&](int c, T val) { dzn[c] = wv[c] - val; }, tcap);
+      with_m(dl, mdl, false, true);
       float v[4] = {-INFINITY, 0.f, -INFINITY, 0.f};
       for (int i = tid; i < n; i += NTHREADS) z[i] = (double)dzn[i];
       for (int i = tid; i < m; i += NTHREADS) nu[i] = (double)dzn[nz + i];
@@ -1699,23 +2033,27 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
       // Residual precision (FP32 factors only): the plain FP32 operator while the previous
       // iteration's μ is above 1e5·mu_tol, the FP64-accurate one from then on.  Convergence
       // is only ever declared on an FP64-accurate residual.
-      bool exact = sizeof(T) == 8;
+      bool exact = sizeof(T) == 8 || WIDE;
       float mu_prev = INFINITY;
       // The KKT residual at the current iterate and its norms (v[0..2]) and μ·p (v[3]).
       auto residual = [&](bool fast, float (&v)[4]) {
         for (int i = tid; i < n + p + m; i += NTHREADS)
           xs[i] = Split<T>::make(i < n ? z[i] : (i < n + p ? lam[i - n] : nu[i - n - p]));
         __syncthreads();
-        if (fast)
-          kkt_apply_fast<T>(n, p, m, Qb, Gb, Ab, xs, tscr, tcap,
-                            [&](int j) { return qd[j]; },
-                            [&](int i) { return s[i] - hd[i]; },
-                            [&](int i) { return -bd[i]; }, rz, rl, rn);
-        else
-          kkt_apply<T>(n, p, m, Qb, Gb, Ab, xs, ascr, kscr,
-                       [&](int j) { return qd[j]; },
-                       [&](int i) { return s[i] - hd[i]; },
-                       [&](int i) { return -bd[i]; }, rz, rl, rn);
+        auto az = [&](int j) { return qd[j]; };
+        auto al = [&](int i) { return s[i] - hd[i]; };
+        auto an = [&](int i) { return -bd[i]; };
+        if constexpr (WIDE) {
+          for (int i = tid; i < n; i += NTHREADS) rz[i] = az(i);
+          for (int i = tid; i < p; i += NTHREADS) rl[i] = al(i);
+          for (int i = tid; i < m; i += NTHREADS) rn[i] = an(i);
+          __syncthreads();
+          // always the FP64-accurate form: the matrices' traffic bounds it
+          dist_kkt<T>(D, n, p, m, Qb, Gb, Ab, xs, rz, rl, rn);
+        } else {
+          if (fast) kkt_apply_fast<T>(n, p, m, Qb, Gb, Ab, xs, tscr, tcap, az, al, an, rz, rl, rn);
+          else kkt_apply<T>(n, p, m, Qb, Gb, Ab, xs, ascr, kscr, az, al, an, rz, rl, rn);
+        }
         v[0] = v[1] = v[2] = v[3] = 0.f;
         for (int i = tid; i < n; i += NTHREADS) v[0] = ropf<R_MAX>(v[0], fabsf((float)rz[i]));
         for (int i = tid; i < p; i += NTHREADS) {
@@ -1780,10 +2118,13 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
           break;
         }
         if (P.time_limit_ns) {
-          if (tid == 0) s_timeout = (globaltimer_ns() - t_start > P.time_limit_ns) ? 1 : 0;
-          __syncthreads();
-          const int out = s_timeout;
-          __syncthreads();
+          // one block decides for the cluster
+          int* flag = D.blocks > 1 ? reinterpret_cast<int*>(D.ex) : &s_timeout;
+          if (tid == 0 && D.rank == 0)
+            *flag = (globaltimer_ns() - t_start > P.time_limit_ns) ? 1 : 0;
+          cluster_barrier(D.blocks);
+          const int out = *flag;
+          cluster_barrier(D.blocks);
           if (out) {
             status = ST_TIMEOUT;
             break;
@@ -1798,13 +2139,11 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
           break;
         }
         // Affine-scaling (predictor) direction, Eq. 9.
-        if (!mv_rows_xreg<8>(SR, ldS, m1 + p, m1, u, [&](int r, T val) { wv[r] = val; }))
-          mv_rows<8>(SR, ldS, m1 + p, m1, TRI_ALL, u, [&](int r, T val) { wv[r] = val; });
-        __syncthreads();
+        with_sr();
         for (int i = tid; i < p; i += NTHREADS) rhsa[i] = wv[m1 + i] + (T)(rl[i] - s[i]);
         __syncthreads();
         solve(rhsa, y, dla, tscr);
-        mv_sym_upper(p, Mb, ldM, dM, dla, tmp, mdl, tscr, tcap);
+        with_m(dla, mdl, true, false);
         // Δs from the complementarity row where s ≤ λ and from the primal row
         // GΔz + Δs = −r_λ (with GΔz = RE·u − MΔλ) elsewhere: the first multiplies the
         // FP32 error of Δλ by s/λ, which is large exactly where the second is safe.
@@ -1838,9 +2177,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         }
         __syncthreads();
         solve(rhs, y, dl, tscr);
-        mv_cols(SR + (size_t)m1 * ldS, ldS, p, m1, TRI_ALL, dl, tscr,
-                [&](int c, T val) { dzn[c] = wv[c] - val; }, tcap);
-        mv_sym_upper(p, Mb, ldM, dM, dl, tmp, mdl, tscr, tcap);
+        with_m(dl, mdl, true, true);
         float w6[4] = {INFINITY, 0.f, 0.f, 0.f};
         for (int i = tid; i < p; i += NTHREADS) {
           const T si = (T)s[i], li = (T)lam[i], d = dl[i];
@@ -1889,6 +2226,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
   // An infeasibility certificate is returned scaled to max(‖λ‖∞, ‖ν‖∞) = 1.
   const double dsc = status == ST_INFEAS ? cert_scale : 1.0;
+  if (D.rank != 0) return;   // every block holds the same iterate
   for (int i = tid; i < n; i += NTHREADS) {
     const double v = bad ? qnan : z[i];
     P.z[i] = (T)v;
@@ -1962,7 +2300,7 @@ __device__ __forceinline__ void fwd_smem_path(const FwdInst<T>& I, unsigned char
   T* cb = reinterpret_cast<T*>(sm + L.ocb);
   const int n = I.n, p = I.p, m = I.m;
   const int tcap = (int)(L.cbytes / sizeof(T));
-  fwd_body<T>(I, L, sm, SR, Mb, L.ldM, dM, false,
+  fwd_body<T, false, false>(I, L, sm, SR, Mb, L.ldM, dM, Dist<T>{1, 0, nullptr, 0},
       [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
         return sweep_setup<T, SW>(n, p, m, Qb, Ab, Gb, SR, L.ldS, Mb, L.ldM, dM, cb, delta, zthr);
       },
@@ -1974,8 +2312,9 @@ __device__ __forceinline__ void fwd_smem_path(const FwdInst<T>& I, unsigned char
 // whether the setup sweep may take its rank-64 updates on the tensor cores (qp_tc.cuh).  The
 // fixed-size kernel does; the persistent packed kernel does not (its tensor-core variant raised
 // a GPU fault whose cause was not found), so its workspace has no panel-tile region.
-template <typename T, bool TC>
-__device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned char* sm) {
+template <typename T, bool TC, bool WIDE>
+__device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned char* sm,
+                                                int blocks, int rank) {
   FwdSmem<T> L;
   L.init(I.n, I.nz, I.p, I.m, true);
   const int n = I.n, p = I.p, m = I.m, nz = I.nz;
@@ -1988,11 +2327,15 @@ __device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned ch
   T* pan = reinterpret_cast<T*>(I.ws + W.oPan);
   T* cb = reinterpret_cast<T*>(sm + L.ocb);
   const int tcap = (int)(L.cbytes / sizeof(T));
-  fwd_body<T>(I, L, sm, SR, Mb, p > 0 ? p : 1, dM, true,
+  // exchange buffer of the cluster's blocks: the panel scratch, idle outside the factorisations
+  // (and in them where the panels are in shared memory)
+  const Dist<T> D{blocks, rank, pan, (int)((W.oTc - W.oPan) / sizeof(T))};
+  fwd_body<T, true, WIDE>(I, L, sm, SR, Mb, p > 0 ? p : 1, dM, D,
       [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
-        return gsweep_setup<T>(n, nz, p, m, Qb, Ab, Gb, SR, Mb, dM, pan, L.span_smem != 0, cb,
+        return gsweep_setup<T, WIDE>(n, nz, p, m, Qb, Ab, Gb, SR, Mb, dM, pan, L.span_smem != 0, cb,
                                delta, zthr,
-                               TC && L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr);
+                               TC && L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr, blocks,
+                               rank);
       },
       [&](const T* dsh) {
         // Small Schur complements: the register-tile routine (M read from and X written to
@@ -2002,7 +2345,7 @@ __device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned ch
         if constexpr (sizeof(T) == 4) {
           if (reg_chol_ok(p, 4)) return chol_blk<T, 2, true>(p, Mb, ldM, dM, dsh, cb);
         }
-        return gchol_factor<T>(p, Mb, dM, dsh, Aw, pan, L.pan_smem != 0, cb);
+        return gchol_factor<T, WIDE>(p, Mb, dM, dsh, Aw, pan, L.pan_smem != 0, cb, pan, blocks, rank);
       },
       [&](const T* rhs, T* y, T* out, T* scr) {
         const int ldM = p > 0 ? p : 1;
@@ -2018,22 +2361,45 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_kernel(const FwdParams<T> 
   fwd_smem_path<T, SW, CH>(fixed_inst(P, blockIdx.x), sm);
 }
 
-// Fixed-size batch, global-memory path.
-template <typename T>
+// Fixed-size batch, global-memory path: P.blocks blocks (a cluster, where more than one) per
+// instance when WIDE, one otherwise.
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_large_kernel(const FwdParams<T> P) {
   extern __shared__ __align__(16) unsigned char sm[];
-  fwd_global_path<T, true>(fixed_inst(P, blockIdx.x), sm);
+  if constexpr (WIDE) {
+    const int inst = (int)blockIdx.x / P.blocks;
+    fwd_global_path<T, true, true>(fixed_inst(P, inst), sm, P.blocks, (int)blockIdx.x - inst * P.blocks);
+  } else {
+    fwd_global_path<T, true, false>(fixed_inst(P, blockIdx.x), sm, 1, 0);
+  }
 }
 
-// Packed batch of uneven sizes, persistent: blocks take instances from an atomic counter in
-// the order of the descriptor array (largest estimated cost first), and each instance runs
-// the path its own size selects, so its result does not depend on the mix.  MODE selects the
-// code compiled in: PK_SMEM the shared-memory path alone (register-allocated on its own, as
-// the fixed-size kernel is), PK_BOTH both paths.  The host runs a batch's global-path
-// instances in a PK_BOTH kernel and its shared-memory-path instances in a PK_SMEM kernel
-// beside it, each over its own descriptor range.
-enum : int { PK_SMEM = 0, PK_BOTH = 1 };
-template <typename T, int SW, int CH, int MODE>
+// Views of a packed batch's instance.
+template <typename T>
+__device__ __forceinline__ FwdInst<T> packed_inst(const PackedFwdParams<T>& P, const PackedDesc& d) {
+  FwdInst<T> I;
+  I.n = d.n; I.p = d.nineq; I.m = d.neq; I.nz = d.nz;
+  I.Q = P.Q + d.oQ; I.q = P.q + d.oq;
+  I.G = d.nineq ? P.G + d.oG : nullptr;
+  I.h = d.nineq ? P.h + d.oh : nullptr;
+  I.A = d.neq ? P.A + d.oA : nullptr;
+  I.b = d.neq ? P.b + d.ob : nullptr;
+  I.z = P.z + d.oz;
+  I.lam = P.lam ? P.lam + d.olam : nullptr;
+  I.nu = P.nu ? P.nu + d.onu : nullptr;
+  I.status = P.status ? P.status + d.id : nullptr;
+  I.iters = P.iters ? P.iters + d.id : nullptr;
+  I.resid = P.resid ? P.resid + 4 * (size_t)d.id : nullptr;
+  I.ws = P.ws + d.ows;
+  I.tol = P.tol; I.mu_tol = P.mu_tol; I.max_iter = P.max_iter;
+  I.time_limit_ns = P.time_limit_ns;
+  return I;
+}
+
+// Shared-memory-path instances of a packed batch of uneven sizes, persistent: blocks take
+// instances from an atomic counter in the order of the descriptor array (largest estimated
+// cost first), so an instance's result does not depend on the mix.
+template <typename T, int SW, int CH>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_kernel(const PackedFwdParams<T> P) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int s_idx;
@@ -2044,39 +2410,37 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_kernel(const Packed
     __syncthreads();
     if (k >= P.B) break;
     const PackedDesc d = P.desc[k];
-    FwdInst<T> I;
-    I.n = d.n; I.p = d.nineq; I.m = d.neq; I.nz = d.nz;
-    I.Q = P.Q + d.oQ; I.q = P.q + d.oq;
-    I.G = d.nineq ? P.G + d.oG : nullptr;
-    I.h = d.nineq ? P.h + d.oh : nullptr;
-    I.A = d.neq ? P.A + d.oA : nullptr;
-    I.b = d.neq ? P.b + d.ob : nullptr;
-    I.z = P.z + d.oz;
-    I.lam = P.lam ? P.lam + d.olam : nullptr;
-    I.nu = P.nu ? P.nu + d.onu : nullptr;
-    I.status = P.status ? P.status + d.id : nullptr;
-    I.iters = P.iters ? P.iters + d.id : nullptr;
-    I.resid = P.resid ? P.resid + 4 * (size_t)d.id : nullptr;
-    I.ws = P.ws + d.ows;
-    I.tol = P.tol; I.mu_tol = P.mu_tol; I.max_iter = P.max_iter;
-    I.time_limit_ns = P.time_limit_ns;
-    const bool glob = (d.flags & 1) != 0;
-    if (glob && MODE == PK_SMEM) {
+    const FwdInst<T> I = packed_inst(P, d);
+    if (d.flags & 1) {
       // Not reached (the host gives each kernel only instances of its own path); should it
       // happen, the instance is marked failed rather than run on the wrong path.
       if (threadIdx.x == 0) {
         WsLayout W;
-        W.init(I.n, I.nz, I.p, I.m, (int)sizeof(T), glob);
+        W.init(I.n, I.nz, I.p, I.m, (int)sizeof(T), true);
         reinterpret_cast<int32_t*>(I.ws + W.oSt)[0] = ST_NUM;
         if (I.status) *I.status = ST_NUM;
       }
-    } else if constexpr (MODE == PK_BOTH) {
-      if (glob) fwd_global_path<T, false>(I, sm);
-      else fwd_smem_path<T, SW, CH>(I, sm);
     } else {
       fwd_smem_path<T, SW, CH>(I, sm);
     }
     __syncthreads();
+  }
+}
+
+// Global-memory-path instances of a packed batch, wide ones (P.blocks blocks, a cluster, where
+// more than one, per instance) or the others, in the order of the descriptor array, largest estimated cost first, which
+// the block scheduler follows.  The setup sweep runs on CUDA cores (its tensor-core form faulted
+// in an earlier persistent form of this kernel, for a reason that was not found).
+template <typename T, bool WIDE>
+__global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_large_kernel(const PackedFwdParams<T> P) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  if constexpr (WIDE) {
+    const int k = (int)blockIdx.x / P.blocks;
+    const PackedDesc d = P.desc[k];
+    fwd_global_path<T, false, true>(packed_inst(P, d), sm, P.blocks, (int)blockIdx.x - k * P.blocks);
+  } else {
+    const PackedDesc d = P.desc[blockIdx.x];
+    fwd_global_path<T, false, false>(packed_inst(P, d), sm, 1, 0);
   }
 }
 

@@ -16,19 +16,16 @@ cudaError_t launch_fwd_large_f32(const FwdParams<float>& P, size_t smem, cudaStr
   return launch_fwd_large_v<float>(P, smem, st);
 }
 
-template <int SW, int CH>
-static cudaError_t gop(const PackedFwdParams<float>& P, size_t smem, int grid, int mode,
-                       cudaStream_t st) {
-  return mode == PK_BOTH ? launch_fwd_packed_v<float, SW, CH, PK_BOTH>(P, smem, grid, st)
-                         : launch_fwd_packed_v<float, SW, CH, PK_SMEM>(P, smem, grid, st);
+cudaError_t launch_fwd_packed_large_f32(const PackedFwdParams<float>& P, size_t smem, cudaStream_t st) {
+  return launch_fwd_packed_large_v<float>(P, smem, st);
 }
 
 cudaError_t launch_fwd_packed_f32(const PackedFwdParams<float>& P, int SW, int CH, size_t smem,
-                                  int grid, int mode, cudaStream_t st) {
-  if (SW == 1 && CH == 1) return gop<1, 1>(P, smem, grid, mode, st);
-  if (SW == 2 && CH == 1) return gop<2, 1>(P, smem, grid, mode, st);
-  if (SW == 4 && CH == 1) return gop<4, 1>(P, smem, grid, mode, st);
-  if (SW == 4 && CH == 2) return gop<4, 2>(P, smem, grid, mode, st);
+                                  int grid, cudaStream_t st) {
+  if (SW == 1 && CH == 1) return launch_fwd_packed_v<float, 1, 1>(P, smem, grid, st);
+  if (SW == 2 && CH == 1) return launch_fwd_packed_v<float, 2, 1>(P, smem, grid, st);
+  if (SW == 4 && CH == 1) return launch_fwd_packed_v<float, 4, 1>(P, smem, grid, st);
+  if (SW == 4 && CH == 2) return launch_fwd_packed_v<float, 4, 2>(P, smem, grid, st);
   return cudaErrorInvalidValue;
 }
 

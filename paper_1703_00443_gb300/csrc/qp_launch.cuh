@@ -23,17 +23,21 @@ template <typename T, int SW, int CH>
 cudaError_t launch_fwd_v(const FwdParams<T>& P, size_t smem, cudaStream_t st);
 template <typename T>
 cudaError_t launch_fwd_large_v(const FwdParams<T>& P, size_t smem, cudaStream_t st);
-template <typename T, int SW, int CH, int MODE>
+template <typename T, int SW, int CH>
 cudaError_t launch_fwd_packed_v(const PackedFwdParams<T>& P, size_t smem, int grid, cudaStream_t st);
+template <typename T>
+cudaError_t launch_fwd_packed_large_v(const PackedFwdParams<T>& P, size_t smem, cudaStream_t st);
 
 cudaError_t launch_fwd_f32(const FwdParams<float>& P, int SW, int CH, size_t smem, cudaStream_t st);
 cudaError_t launch_fwd_f64(const FwdParams<double>& P, int SW, int CH, size_t smem, cudaStream_t st);
 cudaError_t launch_fwd_large_f32(const FwdParams<float>& P, size_t smem, cudaStream_t st);
 cudaError_t launch_fwd_large_f64(const FwdParams<double>& P, size_t smem, cudaStream_t st);
 cudaError_t launch_fwd_packed_f32(const PackedFwdParams<float>& P, int SW, int CH, size_t smem,
-                                  int grid, int mode, cudaStream_t st);
+                                  int grid, cudaStream_t st);
 cudaError_t launch_fwd_packed_f64(const PackedFwdParams<double>& P, int SW, int CH, size_t smem,
-                                  int grid, int mode, cudaStream_t st);
+                                  int grid, cudaStream_t st);
+cudaError_t launch_fwd_packed_large_f32(const PackedFwdParams<float>& P, size_t smem, cudaStream_t st);
+cudaError_t launch_fwd_packed_large_f64(const PackedFwdParams<double>& P, size_t smem, cudaStream_t st);
 cudaError_t launch_bwd_packed_f32(const PackedBwdParams<float>& P, size_t smem, int grid, cudaStream_t st);
 cudaError_t launch_bwd_packed_f64(const PackedBwdParams<double>& P, size_t smem, int grid, cudaStream_t st);
 cudaError_t launch_bwd_f32(const BwdParams<float>& P, size_t smem, cudaStream_t st);

@@ -171,6 +171,27 @@ __device__ __forceinline__ unsigned long long tc_now() {
 }
 #endif  // __CUDA_ARCH__
 
+// Barrier over a thread-block cluster, with everything written to global memory before it
+// visible to every block after it (a cluster of one: a block barrier).
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ void cluster_barrier(int blocks) {
+  if (blocks == 1) {
+    __syncthreads();
+    return;
+  }
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  __threadfence();
+}
+#endif  // __CUDA_ARCH__
+#if !defined(__CUDA_ARCH__)
+__device__ __forceinline__ void cluster_barrier(int blocks) {
+  (void)blocks;
+  __syncthreads();   // a cluster of one
+}
+#endif
+
 // Bounded wait for the completion of phase `parity`; false when TC_WAIT_NS ran out.
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
   if (tc_try_wait(bar, parity)) return true;
@@ -198,10 +219,15 @@ __device__ __forceinline__ float tc_hi(float x) {
 // ldM) plus dM).  `tcp` is the panel-tile region of the workspace, `cb0` the shared work
 // region (≥ TC_SMEM_BYTES, 16-byte aligned).  Pivot sign tests as in gsweep_setup.  Returns
 // false on a pivot that fails its test or on an expired wait.
+template <bool WIDE>
 static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, int m, int nsb,
                                                          float* SR, float* Mb, int ldM, float* dM,
                                                          float* tcp, unsigned char* cb0,
-                                                         float zthr) {
+                                                         float zthr, int blocks, int rank) {
+  if constexpr (!WIDE) {   // one block per instance
+    blocks = 1;
+    rank = 0;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m1 = nz + m, N = m1 + p, ldS = m1;
   const int T1 = (m1 + TC_TM - 1) / TC_TM, T2 = (p + TC_TM - 1) / TC_TM, NT = T1 + T2;
@@ -220,7 +246,8 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
   float* sR = reinterpret_cast<float*>(cb + 16384);            // 64 × 64 multipliers
   uint64_t* bar_mma = reinterpret_cast<uint64_t*>(cb + 4 * TC_TILE_BYTES);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(cb + 4 * TC_TILE_BYTES + 16);
-  int* flag = reinterpret_cast<int*>(cb + 4 * TC_TILE_BYTES + 20);
+  int* flag = reinterpret_cast<int*>(cb + 4 * TC_TILE_BYTES + 20);       // a pivot failed
+  int* late = reinterpret_cast<int*>(cb + 4 * TC_TILE_BYTES + 24);       // a wait expired
 
   // Zero the panel rows past each segment's end (read by the MMA, never stored).
   {
@@ -237,7 +264,7 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
   }
   if (tid == 0) {
     tc_mbar_init(bar_mma);
-    flag[0] = 0;
+    flag[0] = late[0] = 0;
   }
   __syncwarp();
   if (warp == 0) tc_alloc256(tslot);
@@ -247,6 +274,11 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
   const uint32_t tmem = *tslot;
   uint32_t ph_mma = 0;
   bool ok = true;
+  // The blocks of a cluster share the sweep: every block sweeps the pivot block itself, the rows
+  // of phase B and the output tiles of phase C are dealt to the blocks.  A failed pivot is the
+  // same in all; an expired wait is one block's, which skips its tiles from then on but meets
+  // every barrier, and tells the others at the end.
+  bool dead = false;
 
   for (int sb = 0; sb < nsb && ok; ++sb) {
     const int k0 = sb * TC_KB;
@@ -293,16 +325,18 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
         }
         if (rowown) sR[k * TC_KB + pc] = (pc == k) ? dinv : rk * dinv;
       }
-      if (tid == 0) flag[0] = good ? 0 : 1;
+      if (tid == 0 && !good) flag[0] = 1;
       __syncthreads();
       if (flag[0]) { ok = false; break; }
+      if (blocks > 1) cluster_barrier(blocks);   // every block has read the pivot block
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (pr0 + 8 * u < kb && pc < kb) SR[(size_t)(k0 + pr0 + 8 * u) * ldS + k0 + pc] = v[u];
+        if (rank == 0 && pr0 + 8 * u < kb && pc < kb)
+          SR[(size_t)(k0 + pr0 + 8 * u) * ldS + k0 + pc] = v[u];
     }
     // ---- phase B: replay the 64 sweeps on every row outside the superblock; write the
     // panels (p = ĉ/d and c = ĉ, TF32 hi and lo) and the row's superblock entries.
-    for (int i = tid; i < N; i += NTHREADS) {
+    for (int i = rank * NTHREADS + tid; i < N; i += blocks * NTHREADS) {
       if (i >= k0 && i < k0 + kb) continue;
       float* row = SR + (size_t)i * ldS + k0;
       float v[TC_KB];
@@ -361,7 +395,7 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
           if (q < kb) SR[(size_t)(k0 + q) * ldS + i] = v[q];
       }
     }
-    __syncthreads();
+    cluster_barrier(blocks);
     // ---- phase C: the rank-64 update, one 128 × 128 output tile at a time.  SR tiles:
     // row tiles 0..NT−1 (both segments) × column tiles 0..T1−1; λ-by-λ tiles: row tile I ≤
     // column tile J among the T2 λ tiles.  Tile t accumulates in TMEM columns 128·(t & 1);
@@ -376,10 +410,13 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
         ta = T1 + I; tbi = T1 + I + u;
       }
     };
+    // This block's tiles are [tfirst, tend), consecutive so that row tiles repeat.
+    const int tfirst = (int)((long long)ntiles * rank / blocks);
+    const int tend = (int)((long long)ntiles * (rank + 1) / blocks);
     int prevA = -1, pta = 0, ptb = 0;
-    for (int t = 0; t <= ntiles && ok; ++t) {
+    for (int t = tfirst; t <= tend && !dead && tfirst < tend; ++t) {
       int ta = 0, tbi = 0;
-      if (t < ntiles) {
+      if (t < tend) {
         tile_of(t, ta, tbi);
         // stage the operand tiles (A only when the row tile changes); the MMA of tile t − 1
         // has completed, so its operands may be overwritten.  All loads first, then stores.
@@ -427,7 +464,7 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
           tc_commit(bar_mma);
         }
       }
-      if (t > 0) {
+      if (t > tfirst) {
         // epilogue of tile t − 1 (its MMA completed before the last barrier): warp w reads
         // TMEM lanes 32·(w%4)… (tile columns) and TMEM columns 32·(w/4)… (tile rows); lane
         // l holds column 32·(w%4) + l of 32 consecutive rows
@@ -490,20 +527,31 @@ static __device__ __noinline__ bool tc_sweep_superblocks(int n, int nz, int p, i
           }
         }
       }
-      if (t < ntiles) {
-        if (!tc_wait(bar_mma, ph_mma)) atomicExch(flag, 2);
+      if (t < tend) {
+        if (!tc_wait(bar_mma, ph_mma)) atomicExch(late, 1);
         ph_mma ^= 1;
         pta = ta; ptb = tbi;
       }
       // the epilogue's TMEM reads finish before the next MMA reuses its accumulator
       tc_fence_before();
       __syncthreads();
-      if (flag[0]) ok = false;
+      if (late[0]) dead = true;
     }
-    __syncthreads();
+    cluster_barrier(blocks);
+  }
+  if (blocks > 1) {
+    int* word = reinterpret_cast<int*>(tcp);   // the panels are not needed any more
+    cluster_barrier(blocks);
+    if (rank == 0 && tid == 0) word[0] = 0;
+    cluster_barrier(blocks);
+    if (dead && tid == 0) word[0] = 1;
+    cluster_barrier(blocks);
+    if (word[0]) ok = false;
+  } else if (dead) {
+    ok = false;
   }
   // Leave nothing in flight: a failed wait is retried (bounded) before the memory goes.
-  if (tid == 0 && flag[0] == 2) tc_wait(bar_mma, ph_mma ^ 1);
+  if (tid == 0 && late[0]) tc_wait(bar_mma, ph_mma ^ 1);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
