@@ -193,7 +193,7 @@ int qp_backward_ext(const qp_options* opt, int dtype, int B, int n, int nineq, i
                     int32_t* status, void* stream);
 
 /*
- * Packed batches of uneven sizes (one persistent launch each way).
+ * Packed batches of uneven sizes.
  *
  * Instance i has its own (n_i, nineq_i, neq_i); its data are packed back to back in index
  * order in each input buffer (Q_i n_i×n_i row-major, then Q_{i+1}, ...; likewise q, G, h, A,
@@ -206,7 +206,8 @@ typedef struct qp_instance_desc {
   int32_t n, nineq, neq;     /* sizes                                                   */
   int32_t id;                /* index of the instance (status/iters/resid slots)        */
   int32_t nz;                /* n plus dummy padding (set by qp_packed_plan)            */
-  int32_t flags;             /* bit 0: global-memory kernel (set by qp_packed_plan)     */
+  int32_t flags;             /* bit 0: global-memory kernel, bit 1: of a wide size (set
+                                by qp_packed_plan)                                      */
   int64_t oQ, oq, oG, oh, oA, ob;   /* element offsets into the packed inputs/gradients */
   int64_t oz, olam, onu;            /* element offsets into the packed outputs          */
   int64_t ows;                      /* byte offset of the instance's workspace          */
@@ -219,12 +220,14 @@ typedef struct qp_packed_sizes {
   int64_t fwd_smem, bwd_smem;       /* dynamic shared memory of the packed kernels      */
   int32_t sw, ch;                   /* register-tile variant of the shared-memory path  */
   int32_t n_global;                 /* instances on the global-memory path              */
-  int32_t reserved;
+  int32_t reserved;          /* wide instances << 8 | those shared by several blocks; 0:
+                                every global-path instance runs on one block            */
 } qp_packed_sizes;
 
 /* Host-side planning: dims is a HOST array of B triples (n, nineq, neq).  Fills the HOST
- * arrays desc[B] (in execution order: the sizes->n_global global-path instances first, then
- * the shared-memory-path ones, each part largest estimated cost first) and *sizes.  The
+ * arrays desc[B] (in execution order: the sizes->n_global global-path instances first, of
+ * them the wide sizes first, then the shared-memory-path ones, each part largest estimated
+ * cost first) and *sizes.  The
  * caller copies desc to device memory unchanged and passes it, with sizes, to the packed
  * calls. */
 int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
@@ -233,19 +236,19 @@ int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
 /* qp_packed_plan with per-instance hints from a tuner: path_hint[i] (may be NULL) is 0 for
  * the automatic choice, 1 for the global-memory kernel, 2 for the shared-memory kernel
  * (QP_EUNSUPPORTED if it cannot take that size); cost[i] (may be NULL) replaces the built-in
- * cost estimate that orders the work queue (largest first). */
+ * cost estimate that orders the instances (largest first). */
 int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* dims,
                       const int8_t* path_hint, const float* cost, qp_instance_desc* desc,
                       qp_packed_sizes* sizes);
 
 /* Forward pass of a packed batch (device pointers as in qp_forward, packed as above;
- * status/iters/resid indexed by instance id; workspace of sizes->ws_bytes bytes).  When a
- * batch holds both kinds, the global-path and shared-memory-path instances run as two
- * persistent kernels side by side: the global-path one first, on `stream`, the other on a
- * library-owned side stream forked from `stream` and joined back to it by events (one side
- * stream per caller stream, for up to 16 streams per device; created on a stream's first
- * such call: make that call before any stream capture).  Its blocks take SMs as the
- * global-path blocks finish their queue. */
+ * status/iters/resid indexed by instance id; workspace of sizes->ws_bytes bytes).  The
+ * instances shared by several blocks, the other wide ones, the other global-path ones and the
+ * shared-memory-path ones run as up to four kernels side by side: the first on `stream`, the
+ * others on library-owned side streams forked from `stream` and joined back to it by events
+ * (one set per caller stream, for up to 16 streams per device; created on a stream's first
+ * such call: make that call before any stream capture).  Later kernels' blocks take SMs as
+ * the earlier ones' blocks end. */
 int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance_desc* desc,
                       const qp_packed_sizes* sizes, const void* Q, const void* q,
                       const void* G, const void* h, const void* A, const void* b, void* z,

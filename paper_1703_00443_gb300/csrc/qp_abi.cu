@@ -102,7 +102,7 @@ struct Plan {
 };
 
 // force: 0 automatic, 1 global-memory path, 2 shared-memory path (ok = false if impossible).
-// packed: the instance runs in the persistent packed kernel (no tensor-core sweep, so no
+// packed: the instance runs in a packed kernel (no tensor-core sweep, so no
 // panel-tile region in its workspace).
 Plan make_plan(int dtype, int n, int nineq, int neq, int force_global = 0, bool packed = false) {
   Plan pl;
@@ -208,9 +208,16 @@ double est_cost(int n, int nz, int p, int m, bool large) {
   return large ? 3.0 * c : c;
 }
 
-// Blocks per instance on the global-memory path for a batch of B: a cluster of up to eight while
-// the whole batch's clusters are resident at once (one block per SM; a cluster needs its SMs
-// within one processing cluster of 16 to 20, which leaves a few SMs unused), one block otherwise.
+// Blocks per instance of a wide size for a batch of B: a cluster of up to eight while the whole
+// batch's clusters are resident at once (one block per SM; a cluster needs its SMs within one
+// processing cluster of 16 to 20, which leaves a few SMs unused), one block otherwise.  The
+// shares taken of the SMs (3/4 for clusters of eight, 9/10 for the others) are that
+// fragmentation.  One n = 500 instance, forward and backward: 25.9 ms on one block of the
+// one-block kernels, 12.9 ms on eight; what is left is the chains that every block waits for.
+// The leading instances of a packed batch take at least kQueuedBlocks each, also when their
+// clusters have to take turns: 256 mixed requests with 72 such instances took 31.9 ms at one
+// block each before clusters, 21.9 ms now; the resident rule alone leaves
+// them at one block each.
 #if defined(QP_HOST_EMULATION)
 constexpr int kQueuedBlocks = 1;
 #else
@@ -442,7 +449,8 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   S.sw = sw; S.ch = ch;
   // Wide instances to share among several blocks: the leading ones (largest first) whose own
   // estimated time on one SM would exceed 1.2 of the batch's total over all SMs, and so set
-  // the batch's time.  The plan keeps both counts in `reserved`.
+  // the batch's time: sharing more of them only takes SMs from whole instances, which use them
+  // better.  The plan keeps both counts in `reserved`.
   double total = 0.0;
   for (const auto& x : order) total += x.first;
   const double limit = 1.2 * total / num_sms();
@@ -512,8 +520,8 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
   int np = 0;
   const int nwide = std::min(std::max(sizes->reserved >> 8, 0), ng);
   const int nshare = std::min(sizes->reserved & 255, nwide);
-  // (four blocks each where the clusters take turns)
-  if (nshare > 0) parts[np++] = {std::max(blocks_per_instance(nshare, true), kQueuedBlocks), 0, nshare};
+  if (nshare > 0)
+    parts[np++] = {std::max(blocks_per_instance(nshare, true), kQueuedBlocks), 0, nshare};
   if (nwide > nshare) parts[np++] = {1, nshare, nwide - nshare};
   if (ng > nwide) parts[np++] = {0, nwide, ng - nwide};
   if (ns > 0) parts[np++] = {-1, ng, ns};
@@ -522,7 +530,12 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
     return e == cudaSuccess ? QP_OK : QP_ECUDA;
   }
   SideStream* ss = side_stream(st);
-  if (!ss) return QP_ECUDA;
+  if (!ss) {   // no side streams to be had: one after the other
+    bool ok = true;
+    for (int i = 0; i < np; ++i)
+      ok = launch(parts[i].kind, parts[i].off, parts[i].cnt, st) == cudaSuccess && ok;
+    return ok ? QP_OK : QP_ECUDA;
+  }
   std::lock_guard<std::mutex> lk(ss->mu);
   if (cudaEventRecord(ss->fork, st) != cudaSuccess) return QP_ECUDA;
   if (launch(parts[0].kind, parts[0].off, parts[0].cnt, st) != cudaSuccess) return QP_ECUDA;

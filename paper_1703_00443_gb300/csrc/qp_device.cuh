@@ -960,7 +960,9 @@ struct Dist {
 };
 
 // Sizes that take these products: below them one block's registers and its own shared-memory
-// partial sums are faster (n = 200, nineq = 150: 2.6 ms a batch of 128 against 4.3).
+// partial sums are faster (n = 200, nineq = 150: 2.6 ms a batch of 128 against 4.3), and a
+// cluster gains little, since the panel and pivot chains are the larger part there (a line at
+// n + neq or nineq of 320 made a batch of 512 uneven instances 7% slower).
 __host__ __device__ inline bool wide_size(int m1) { return m1 >= 352; }
 
 // out[r] = Σ_c M[r·ld + c]·x[c] over all c < cols (upper = false) or c > r, eight lanes per row,
@@ -2427,9 +2429,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_kernel(const Packed
   }
 }
 
-// Global-memory-path instances of a packed batch, wide ones (P.blocks blocks, a cluster, where
-// more than one, per instance) or the others, in the order of the descriptor array, largest estimated cost first, which
-// the block scheduler follows.  The setup sweep runs on CUDA cores (its tensor-core form faulted
+// Global-memory-path instances of a packed batch, wide ones (P.blocks blocks per instance, a
+// cluster where more than one) or the others, in the order of the descriptor array (largest
+// estimated cost first), which the block scheduler follows: no work queue, and no second
+// path's code and spills in the kernel.  Bound by the longest instance's chain, then by the L2
+// traffic of the factors of 152 instances in flight.  512 uneven instances, forward and
+// backward: 17.4 ms with a persistent kernel of both paths, 16.9 ms now.  The setup sweep runs on CUDA cores (its tensor-core form faulted
 // in an earlier persistent form of this kernel, for a reason that was not found).
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_large_kernel(const PackedFwdParams<T> P) {

@@ -4,8 +4,12 @@
 // Mb plus dM, the Cholesky factor in the lower triangle of Mb), but the matrices live in the instance's
 // global workspace (L2-resident during the solve).  Pivots are taken in blocks: one warp
 // handles the pivot block, all threads then form the panel and apply the rank-block update
-// to the trailing matrix (LNB = 16 columns per block in the setup sweep, chol_nb columns in
-// the per-iteration Cholesky, whose current block column and panel stay in shared memory).
+// to the trailing matrix (LNB = 16 columns per block in the setup sweep, 32 or 16 in the
+// per-iteration Cholesky, whose current block column and panel stay in shared memory).
+// A wide size may be shared by the blocks of a cluster.  Each of them forms the whole panel
+// in its own shared memory (p = 500: about 200K cycles for all of a factorisation's panels)
+// and takes its share of the trailing update; a cluster barrier a block
+// column is the only meeting point.
 #pragma once
 
 namespace qpk {
@@ -338,13 +342,16 @@ __device__ __noinline__ void gchol_pivot_block(int k0, int nb, const T* Sb, int 
 //   A: warp 0 factors the diagonal block from S (gchol_pivot_block);
 //   B: one thread per row i ≥ t0 solves L_KK l_iᵀ = a_iᵀ (row i of the panel L_IK) by forward
 //      substitution, shifting the row through registers so the results come out in order;
-//      P[c][i] and Mb[i][k0 + c] receive it;
+//      P[c][i] and Mb[i][k0 + c] receive it.  NB more items solve for the unit vectors: the
+//      columns of V_K;
 //   C: every lower-triangle entry of the trailing matrix takes A_IJ −= L_IK L_JKᵀ in 8×4
 //      register micro-tiles (tile row t0/8 + R holds the 2R + 2 tiles of columns
 //      t0..t0+8R+7).  Tiles of block column K + 1 go to S instead of Aw: they are final and
-//      only the next pivot block and panel read them.  Meanwhile warp 0 takes the tiles of the
-//      next diagonal block and then runs step A of block K + 1 (the pivot columns are
-//      double-buffered by block parity).
+//      only the next pivot block and panel read them.  The tiles of the next diagonal block
+//      come first, by all threads; then warp 0 runs step A of block K + 1 while the others go
+//      on (the pivot columns are double-buffered by block parity).
+// Bound by the chain pivot block, panel, diagonal tiles.  p = 500: 1.34M cycles a
+// factorisation before the pivot block was cut to 4.8K cycles, 0.65M now on eight blocks.
 // NB is 32 for FP32 and 16 for FP64 (register room of the pivot block).  Returns false on
 // every thread on a non-positive pivot.
 // WIDE: as in gsweep_setup; Sx is then the workspace's exchange buffer.
