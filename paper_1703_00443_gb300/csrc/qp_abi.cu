@@ -151,8 +151,8 @@ static_assert(sizeof(qp_instance_desc) == sizeof(qpk::PackedDesc), "descriptor l
 struct SideStream {
   cudaStream_t owner = nullptr;   // the caller stream this slot serves
   bool used = false;
-  cudaStream_t s[3] = {nullptr, nullptr, nullptr};
-  cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
+  cudaStream_t s[5] = {};
+  cudaEvent_t fork = nullptr, join[5] = {};
   std::mutex mu;
 };
 constexpr int kSideSlots = 16;
@@ -175,7 +175,7 @@ SideStream* side_stream(cudaStream_t owner) {
   if (!x) x = &row[(reinterpret_cast<uintptr_t>(owner) >> 4) % kSideSlots];
   if (!x->used) {
     bool ok = x->fork || cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 5; ++i) {
       ok = ok && (x->s[i] || cudaStreamCreateWithFlags(&x->s[i], cudaStreamNonBlocking) == cudaSuccess);
       ok = ok && (x->join[i] ||
                   cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess);
@@ -214,15 +214,6 @@ double est_cost(int n, int nz, int p, int m, bool large) {
 // shares taken of the SMs (3/4 for clusters of eight, 9/10 for the others) are that
 // fragmentation.  One n = 500 instance, forward and backward: 25.9 ms on one block of the
 // one-block kernels, 12.9 ms on eight; what is left is the chains that every block waits for.
-// The leading instances of a packed batch take at least kQueuedBlocks each, also when their
-// clusters have to take turns: 256 mixed requests with 72 such instances took 31.9 ms at one
-// block each before clusters, 21.9 ms now; the resident rule alone leaves
-// them at one block each.
-#if defined(QP_HOST_EMULATION)
-constexpr int kQueuedBlocks = 1;
-#else
-constexpr int kQueuedBlocks = 4;
-#endif
 int blocks_per_instance(int B, bool share) {
 #if defined(QP_HOST_EMULATION)
   return 1;   // the host emulation runs one block at a time
@@ -233,6 +224,22 @@ int blocks_per_instance(int B, bool share) {
   if (B * 4 <= nsm * 9 / 10) return 4;
   if (B * 2 <= nsm * 9 / 10) return 2;
   return 1;
+}
+
+// Blocks of the leading `nshare` wide instances of a packed batch, largest first: all of them
+// resident at once, so two blocks each, then four for as many as the SMs hold, then eight.
+// Clusters that wait for their turn cost more than they give (256 mixed requests, 46 shared: at
+// four blocks each 21.1 ms, at four and two all resident 17.6), and blocks left idle are worth
+// most to the largest (96 requests, 24 shared: at four 15.4 ms, the first ten at eight 13.0).
+struct Levels { int n8, n4, n2; };   // instances at eight, four and two blocks, in this order
+Levels share_levels(int nshare) {
+  const int nsm = num_sms(), most = nsm * 9 / 10;
+  nshare = std::min(nshare, most / 2);
+  int left = most - 2 * nshare;
+  const int n48 = std::min(nshare, left / 2);
+  left -= 2 * n48;
+  const int n8 = std::min({n48, left / 4, nsm * 3 / 4 / 8});
+  return {n8, n48 - n8, nshare - n48};
 }
 
 namespace qpk {
@@ -447,18 +454,22 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   S.ws_bytes = ows;
   S.fwd_smem = (int64_t)fsm; S.bwd_smem = (int64_t)bsm;
   S.sw = sw; S.ch = ch;
-  // Wide instances to share among several blocks: the leading ones (largest first) whose own
+  // Wide instances to share among several blocks: leading ones (largest first) whose own
   // estimated time on one SM would exceed 1.2 of the batch's total over all SMs, and so set
   // the batch's time: sharing more of them only takes SMs from whole instances, which use them
-  // better.  The plan keeps both counts in `reserved`.
+  // better.  Where four blocks each would hold nearly all SMs, the last few stay on one, so
+  // that six have eight: they would wait for the first otherwise (128 requests: 33 shared
+  // 15.7 ms, 28 shared 13.3).  The plan keeps both counts in `reserved`.
   double total = 0.0;
   for (const auto& x : order) total += x.first;
   const double limit = 1.2 * total / num_sms();
-  while (nshare < std::min(nwide, 255) && order[nshare].first > limit) {
+  const int budget = num_sms() * 9 / 10;
+  while (nshare < std::min({nwide, 255, budget / 2}) && order[nshare].first > limit) {
     const qp_instance_desc& d = desc[nshare];
     if (!panels_in_smem(dtype, d.n, d.nz, d.nineq, d.neq)) break;
     ++nshare;
   }
+  if (4 * nshare <= budget) nshare = std::min(nshare, std::max(budget / 4 - 6, 0));
   S.reserved = nwide << 8 | nshare;
   *sizes = S;
   return QP_OK;
@@ -509,20 +520,31 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
                 : qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem,
                                              grid, s);
   };
-  // Up to four kernels side by side: the largest wide instances with several blocks each (first
-  // in the descriptor array), the other wide ones, the other global-path ones, and the
+  // Up to six kernels side by side: the largest wide instances with eight, four and two blocks
+  // each (first in the descriptor array), the other wide ones, the other global-path ones, and the
   // shared-memory-path ones; the first of them on `stream`, the others on side streams forked
   // from it and joined back to it, launched in this order so that the costliest take the SMs
   // first.  A block holds its SM until it ends (the last kernel's until its queue runs dry), so
   // as blocks finish, the next kernel's take their SMs: the hardware block scheduler
   // balances the queues without a fixed split.
-  struct Part { int kind, off, cnt; } parts[4];
+  struct Part { int kind, off, cnt; } parts[6];
   int np = 0;
   const int nwide = std::min(std::max(sizes->reserved >> 8, 0), ng);
   const int nshare = std::min(sizes->reserved & 255, nwide);
-  if (nshare > 0)
-    parts[np++] = {std::max(blocks_per_instance(nshare, true), kQueuedBlocks), 0, nshare};
-  if (nwide > nshare) parts[np++] = {1, nshare, nwide - nshare};
+#if defined(QP_HOST_EMULATION)
+  const Levels lv{0, 0, 0};   // the host emulation runs one block at a time
+#else
+  const Levels lv = share_levels(nshare);
+#endif
+  int off = 0;
+  auto add = [&](int kind, int cnt) {
+    if (cnt > 0) parts[np++] = {kind, off, cnt};
+    off += cnt;
+  };
+  add(8, lv.n8);
+  add(4, lv.n4);
+  add(2, lv.n2);
+  add(1, nwide - off);
   if (ng > nwide) parts[np++] = {0, nwide, ng - nwide};
   if (ns > 0) parts[np++] = {-1, ng, ns};
   if (np == 1) {
