@@ -107,6 +107,20 @@ __host__ __device__ inline bool tc_sweep_ok(int n, int nz, int p, int m, int esz
          TC_SMEM_BYTES + large_tail_bytes(n, p, m, m1, 4) <= TC_SMEM_CAP;
 }
 
+// Sizes of the global-memory path whose products are dealt to the blocks of a cluster (Dist).  A full
+// batch, one block each, forward ms with the products of the other sizes and with these, batch 128
+// (n, nineq, neq): (352, 20, 0) 2.48 and 2.15, (352, 176, 0) 5.01 and 4.83, (288, 120, 64) 3.36 and
+// 3.17, (500, 20, 0) 4.07 and 3.74, (500, 500, 125) 33.8 and 27.8; one instance, on eight blocks,
+// 1.76 and 1.29 to 22.4 and 10.4.  Below the line a cluster gained little when it was drawn, since the
+// panel and pivot chains are the larger part there (a line at n + neq or nineq of 320 made a
+// batch of 512 uneven instances 7% slower).
+__host__ __device__ inline bool wide_size(int m1) { return m1 >= 352; }
+
+// The dealt products' copies ahead: 16-byte slots per thread in the shared work region, in batches of
+// half of them.
+constexpr int RING_SLOTS = 8, RING_BATCH = RING_SLOTS / 2;
+constexpr size_t RING_BYTES = RING_SLOTS * 16 * NTHREADS;
+
 // Number of primal variables after padding: 0-3 decoupled dummy variables (Q = 1 on the
 // diagonal, no constraint coupling) make n + neq a multiple of 4, so the pivot blocks of
 // the setup sweep are whole 4×4 tiles.  Dummies sit after the real z entries and stay 0.
@@ -153,7 +167,7 @@ struct WsLayout {
 // Dynamic shared memory of the forward kernel.
 template <typename T>
 struct FwdSmem {
-  int nz, m1, N3, ldS, ldM, NT3, NTp, pan_smem, span_smem, tc_sweep;
+  int nz, m1, N3, ldS, ldM, NT3, NTp, pan_smem, span_smem, tc_sweep, ring;
   size_t oSR, oMb, odM, ocb, cbytes, odbl, osplit, ovec, ored, total;
   // large: S/RE, M/X and diag(M) live in the global workspace, only vectors and a work
   // region stay in shared memory.
@@ -193,7 +207,7 @@ struct FwdSmem {
       }
       cbytes = align_up(c, 16);
     }
-    pan_smem = span_smem = tc_sweep = 0;
+    pan_smem = span_smem = tc_sweep = ring = 0;
     const size_t p4 = (size_t)(p + 3) / 4 * 4;
     const size_t tail = large_tail_bytes(n, p, m, m1, es);
     if (large) {
@@ -218,6 +232,9 @@ struct FwdSmem {
         tc_sweep = 1;
         if (TC_SMEM_BYTES > cbytes) cbytes = align_up(TC_SMEM_BYTES, 16);
       }
+      // Room for the dealt products' copies, if it fits.
+      ring = wide_size(m1) && o + (cbytes > RING_BYTES ? cbytes : RING_BYTES) + tail <= LARGE_PANEL_SMEM_CAP;
+      if (ring && RING_BYTES > cbytes) cbytes = RING_BYTES;
     }
     o += cbytes;
     odbl = o;  o = align_up(o + 8 * (3 * (size_t)n + 4 * (size_t)p + 3 * (size_t)m), 16);
@@ -945,6 +962,15 @@ __device__ __forceinline__ void kkt_apply_fast(int n, int p, int m, const T* __r
   __syncthreads();
 }
 
+// Asynchronous 16-byte copy global → shared (cp.async), and the wait for all of a thread's.
+__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(s), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ products over a cluster
 // The global-memory path may run an instance on a cluster of several blocks: each block keeps
 // the vectors and takes every scalar decision itself, on identical values, and the blocks
@@ -957,69 +983,120 @@ struct Dist {
   int blocks, rank;
   T* ex;          // exchange buffer (workspace)
   int cap;        // its size in elements of T
+  unsigned char* ring;   // RING_BYTES bytes of the shared work region, or null where it has not got them
+  int rest;              // bytes of the shared work region after the ring
 };
 
-// Sizes that take these products: below them one block's registers and its own shared-memory
-// partial sums are faster (n = 200, nineq = 150: 2.6 ms a batch of 128 against 4.3), and a
-// cluster gains little, since the panel and pivot chains are the larger part there (a line at
-// n + neq or nineq of 320 made a batch of 512 uneven instances 7% slower).
-__host__ __device__ inline bool wide_size(int m1) { return m1 >= 352; }
+// The products' matrices come from L2 or HBM, and a shared work region near the limit leaves the
+// L1 less room than the loads in flight need.  So each thread copies its own vectors ahead with
+// cp.async, into RING_SLOTS slots of 16 bytes of its own (no barriers, no registers): batches of
+// half the slots, one of them on its way while the other is summed.  Cycles of the product with
+// [S; RE] in a full batch of 128, with eight 16-byte loads in registers and with the slots: n = 352,
+// nineq = 20 54K and 23K, n = 500, nineq = 20 100K and 45K, n = nineq = 500, neq = 125 244K and 86K
+// (26 bytes a cycle and SM: the copy bandwidth of the 128 SMs); of the residual 103K and 51K, 161K
+// and 89K, 552K and 342K.
+__device__ __forceinline__ unsigned char* ring_slot(unsigned char* ring, int k) {
+  return ring + ((size_t)k * NTHREADS + threadIdx.x) * 16;
+}
+__device__ __forceinline__ void ld16(float (&v)[4], const unsigned char* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void ld16(double (&v)[2], const unsigned char* p) {
+  const double2 t = *reinterpret_cast<const double2*>(p);
+  v[0] = t.x; v[1] = t.y;
+}
 
 // out[r] = Σ_c M[r·ld + c]·x[c] over all c < cols (upper = false) or c > r, eight lanes per row,
-// for the rows dealt to this block.  x is shared memory.  No barrier inside.  Loads go in
-// batches of eight per lane with the tail masked: a remainder loop would wait for L2 one load
-// after the other.
+// for the rows dealt to this block.  x is shared memory.  No barrier inside.  The order of the sums
+// is that of the lanes' vectors, whichever way they are loaded.
 template <typename T>
 __device__ __noinline__ void dist_rows(const Dist<T>& D, const T* M, int ld, int rows, int cols,
                                           bool upper, const T* x, T* out) {
-  constexpr int GL = 8, NG = NTHREADS / GL, W = 16 / sizeof(T);
-  const int g = threadIdx.x / GL, gl = threadIdx.x % GL;
+  constexpr int GL = 8, NG = NTHREADS / GL, W = 16 / sizeof(T), U = RING_BATCH, CS = GL * W * U;
+  const int g = threadIdx.x / GL, gl = threadIdx.x % GL, step = D.blocks * NG;
   const bool vec = !upper && ld % W == 0 && cols % W == 0;
+  unsigned char* ring = D.ring;
+  if (vec && ring != nullptr) {
+    int pr = D.rank * NG + g, pc = W * gl, pb = 0;   // the next batch to copy: row, column, half
+    auto issue = [&]() {
+      if (pr < rows) {
+        const T* src = M + (size_t)pr * ld;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (pc + GL * W * u < cols) cp_async16(ring_slot(ring, pb + u), src + pc + GL * W * u);
+        pc += CS;
+        if (pc >= cols) {
+          pc = W * gl;
+          pr += step;
+        }
+        pb ^= U;
+      }
+      cp_async_commit();
+    };
+    issue();
+    int cb = 0;
 #pragma unroll 1
-  for (int r0 = D.rank * NG; r0 < rows; r0 += D.blocks * NG) {
+    for (int r0 = D.rank * NG; r0 < rows; r0 += step) {
+      const int r = r0 + g;
+      T a0 = T(0), a1 = T(0);
+      if (r < rows) {
+#pragma unroll 1
+        for (int c0 = W * gl; c0 < cols; c0 += CS) {
+          issue();
+          cp_async_wait_but_one();
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int c = c0 + GL * W * u;
+            if (c < cols) {
+              T a[W], xv[W];
+              ld16(a, ring_slot(ring, cb + u));
+              ld16(xv, reinterpret_cast<const unsigned char*>(x + c));
+#pragma unroll
+              for (int e = 0; e < W; ++e) {
+                if (e & 1) a1 = fma(a[e], xv[e], a1);
+                else a0 = fma(a[e], xv[e], a0);
+              }
+            }
+          }
+          cb ^= U;
+        }
+      }
+      T s = a0 + a1;
+#pragma unroll
+      for (int off = GL / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      if (r < rows && gl == 0) out[r] = s;
+    }
+    cp_async_wait_all();
+    return;
+  }
+#pragma unroll 1
+  for (int r0 = D.rank * NG; r0 < rows; r0 += step) {
     const int r = r0 + g;
     const T* row = M + (size_t)r * ld;
     T a0 = T(0), a1 = T(0);
     if (r < rows) {
       if (vec) {
-        constexpr int U = 8;
 #pragma unroll 1
-        for (int cb = W * gl; cb < cols; cb += GL * W * U) {
-          T a[U][W];
+        for (int cb = W * gl; cb < cols; cb += GL * W) {
+          T a[W], xv[W];
+          ld16(a, reinterpret_cast<const unsigned char*>(row + cb));
+          ld16(xv, reinterpret_cast<const unsigned char*>(x + cb));
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int c = cb + GL * W * u;
-            if constexpr (W == 4) {
-              const float4 t = c < cols ? *reinterpret_cast<const float4*>(row + c)
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-              a[u][0] = t.x; a[u][1] = t.y; a[u][2] = t.z; a[u][3] = t.w;
-            } else {
-              const double2 t = c < cols ? *reinterpret_cast<const double2*>(row + c)
-                                         : make_double2(0.0, 0.0);
-              a[u][0] = t.x; a[u][1] = t.y;
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int c = cb + GL * W * u;
-            if (c < cols) {
-#pragma unroll
-              for (int e = 0; e < W; ++e) {
-                if (e & 1) a1 = fma(a[u][e], x[c + e], a1);
-                else a0 = fma(a[u][e], x[c + e], a0);
-              }
-            }
+          for (int e = 0; e < W; ++e) {
+            if (e & 1) a1 = fma(a[e], xv[e], a1);
+            else a0 = fma(a[e], xv[e], a0);
           }
         }
       } else {
-        constexpr int U = 16;
+        constexpr int V = 16;   // loads in flight, the last batch's tail masked
 #pragma unroll 1
-        for (int cb = (upper ? r + 1 : 0) + gl; cb < cols; cb += GL * U) {
-          T a[U];
+        for (int cb = (upper ? r + 1 : 0) + gl; cb < cols; cb += GL * V) {
+          T a[V];
 #pragma unroll
-          for (int u = 0; u < U; ++u) a[u] = cb + GL * u < cols ? row[cb + GL * u] : T(0);
+          for (int u = 0; u < V; ++u) a[u] = cb + GL * u < cols ? row[cb + GL * u] : T(0);
 #pragma unroll
-          for (int u = 0; u < U; ++u)
+          for (int u = 0; u < V; ++u)
             if (cb + GL * u < cols) a0 = fma(a[u], x[cb + GL * u], a0);
         }
       }
@@ -1064,14 +1141,14 @@ __device__ __noinline__ void dist_cols(const Dist<T>& D, const T* M, int ld, int
         const int r1 = upper ? min(rend, c + 3) : rend;   // rows < some column of the four
         float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-        for (int r = r0; r < r1; r += 8) {
-          float4 v[8];
+        for (int r = r0; r < r1; r += 4) {
+          float4 v[4];
 #pragma unroll
-          for (int u = 0; u < 8; ++u)
+          for (int u = 0; u < 4; ++u)
             v[u] = r + u < r1 ? *reinterpret_cast<const float4*>(M + (size_t)(r + u) * ld + c)
                               : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int u = 0; u < 8; ++u)
+          for (int u = 0; u < 4; ++u)
             if (r + u < r1) {
               const float t = x[r + u];
               // (upper: entries on and below the diagonal belong to the factor)
@@ -1125,88 +1202,170 @@ __device__ __forceinline__ int dist_kkt_parts(int n, int R, size_t bytes) {
   const int nq = (n + 3) >> 2;
   return max(1, min((R + 31) >> 5, (int)(bytes / (8 * 4 * (size_t)nq))));
 }
+// The two passes; RING: the rows' quads are copied ahead into the ring (rows on 16-byte boundaries),
+// else loaded where they are used (the values and the order of the sums are the same).
+template <bool RING, typename T>
+__device__ __forceinline__ void dist_kkt_passes(const Dist<T>& D, int n, int p, int m, const T* Q,
+                                                const T* G, const T* A,
+                                                const typename Split<T>::V* xv, Acc<T>* rowres,
+                                                Acc<T>* parts, int nparts, bool vec) {
+  using V = typename Split<T>::V;
+  using AC = Acc<T>;
+  constexpr int QS = sizeof(T) / 4;   // slots of a quad
+  const int tid = threadIdx.x, R = n + p + m, nq = (n + 3) >> 2;
+  const int chunk = (R + nparts - 1) / nparts;
+  unsigned char* ring = D.ring;
+  auto copy = [&](int slot, const T* src) {
+    cp_async16(ring_slot(ring, slot), src);
+    if constexpr (QS == 2) cp_async16(ring_slot(ring, slot + 1), src + 2);
+  };
+  auto quad = [&](T (&v)[4], int slot) {
+    if constexpr (QS == 1) {
+      ld16(v, ring_slot(ring, slot));
+    } else {
+      T a[2], b[2];
+      ld16(a, ring_slot(ring, slot));
+      ld16(b, ring_slot(ring, slot + 1));
+      v[0] = a[0]; v[1] = a[1]; v[2] = b[0]; v[3] = b[1];
+    }
+  };
+  // column pass: quads of columns over row ranges
+#pragma unroll 1
+  for (int t = D.rank * NTHREADS + tid; t < nq * nparts; t += D.blocks * NTHREADS) {
+    const int part = t / nq, jq = t - part * nq;
+    const int r0 = part * chunk, r1 = min(R, r0 + chunk);
+    constexpr int RB = RING_BATCH / QS;
+    AC acc[4];
+#pragma unroll 1
+    for (int seg = 0; seg < 3; ++seg) {   // the rows of Q, G and A
+      const int s0 = seg == 0 ? 0 : (seg == 1 ? n : n + p);
+      const int rs = max(r0, s0), re = min(r1, seg == 0 ? n : (seg == 1 ? n + p : R));
+      if (rs >= re) continue;
+      const T* src = (seg == 0 ? Q : (seg == 1 ? G : A)) + ((size_t)(rs - s0) * n + 4 * jq);
+      int rc = rs, half = 0;   // the next row to copy
+      auto issue = [&](int h) {
+#pragma unroll
+        for (int u = 0; u < RB; ++u)
+          if (rc + u < re) copy(h + QS * u, src + (size_t)(rc + u - rs) * n);
+        rc += RB;
+        cp_async_commit();
+      };
+      if constexpr (RING) issue(0);
+#pragma unroll 1
+      for (int r = rs; r < re; r += RB) {
+        T av[RB][4];
+        if constexpr (RING) {
+          issue(half ^ RING_BATCH);
+          cp_async_wait_but_one();
+        }
+#pragma unroll
+        for (int u = 0; u < RB; ++u)
+          if (r + u < re) {
+            if constexpr (RING) quad(av[u], half + QS * u);
+            else ldg4_row(av[u], src + (size_t)(r + u - rs) * n - 4 * jq, 4 * jq, n, vec);
+          }
+#pragma unroll
+        for (int u = 0; u < RB; ++u)
+          if (r + u < re) {
+            const V x = xv[r + u];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c].add(av[u][c], x);
+          }
+        half ^= RING_BATCH;
+      }
+      if constexpr (RING) cp_async_wait_all();
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) parts[(size_t)part * 4 * nq + 4 * jq + c] = acc[c];
+  }
+  // row pass: eight lanes per row, two rows per lane group; the last blocks and warps take the
+  // first rows, since the first have the more items of the column pass
+  constexpr int GL = 8, NG = NTHREADS / GL, QB = RING_BATCH / (2 * QS);
+  const int g = NG - 1 - tid / GL, gl = tid % GL, rows = p + m;
+#pragma unroll 1
+  for (int r0 = (D.blocks - 1 - D.rank) * 2 * NG; r0 < rows; r0 += D.blocks * 2 * NG) {
+    if (r0 + (NWARPS - 1 - (tid >> 5)) * (32 / GL) >= rows) continue;   // no row for this warp
+    const bool two = r0 + NG < rows;
+    const int rr[2] = {r0 + g, r0 + NG + g};
+    const T* rowv[2];
+#pragma unroll
+    for (int h2 = 0; h2 < 2; ++h2) {
+      const int r = min(rr[h2], rows - 1);
+      rowv[h2] = r < p ? G + (size_t)r * n : A + (size_t)(r - p) * n;
+    }
+    int qc = gl, half = 0;   // the next quad to copy
+    auto issue = [&](int h) {
+#pragma unroll
+      for (int u = 0; u < QB; ++u)
+        if (qc + u * GL < nq) {
+          copy(h + 2 * QS * u, rowv[0] + 4 * (qc + u * GL));
+          if (two) copy(h + 2 * QS * u + QS, rowv[1] + 4 * (qc + u * GL));
+        }
+      qc += GL * QB;
+      cp_async_commit();
+    };
+    if constexpr (RING) issue(0);
+    AC acc[2];
+#pragma unroll 1
+    for (int q0 = gl; q0 < nq; q0 += GL * QB) {
+      T av[2][QB][4];
+      if constexpr (RING) {
+        issue(half ^ RING_BATCH);
+        cp_async_wait_but_one();
+      }
+#pragma unroll
+      for (int u = 0; u < QB; ++u) {
+        const int q = q0 + u * GL;
+        if (q < nq) {
+#pragma unroll
+          for (int h2 = 0; h2 < 2; ++h2)
+            if (h2 == 0 || two) {
+              if constexpr (RING) quad(av[h2][u], half + 2 * QS * u + QS * h2);
+              else ldg4_row(av[h2][u], rowv[h2], 4 * q, n, vec);
+            }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < QB; ++u) {
+        const int q = q0 + u * GL;
+        if (q < nq) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (RING || 4 * q + c < n) {
+              const V x = xv[4 * q + c];
+              acc[0].add(av[0][u][c], x);
+              if (two) acc[1].add(av[1][u][c], x);
+            }
+        }
+      }
+      half ^= RING_BATCH;
+    }
+    if constexpr (RING) cp_async_wait_all();
+#pragma unroll
+    for (int h2 = 0; h2 < 2; ++h2) {
+#pragma unroll
+      for (int off = GL / 2; off > 0; off >>= 1) acc[h2].shfl_merge(off);
+      if (rr[h2] < rows && gl == 0) rowres[rr[h2]] = acc[h2];
+    }
+  }
+}
 template <typename T>
 __device__ __noinline__ void dist_kkt(const Dist<T>& D, int n, int p, int m,
                                          const T* __restrict__ Q, const T* __restrict__ G,
                                          const T* __restrict__ A, const typename Split<T>::V* xv,
                                          double* out_z, double* out_l, double* out_n) {
-  using V = typename Split<T>::V;
   using AC = Acc<T>;
   const int tid = threadIdx.x, R = n + p + m, nq = (n + 3) >> 2;
   const bool vec = (n % 4 == 0) &&
       ((((uintptr_t)Q) | ((uintptr_t)G) | ((uintptr_t)A)) % (4 * sizeof(T)) == 0);
-  auto rowp = [&](int r) -> const T* {
-    return r < n ? Q + (size_t)r * n : (r < n + p ? G + (size_t)(r - n) * n : A + (size_t)(r - n - p) * n);
-  };
-  AC* rowres = reinterpret_cast<AC*>(D.ex);
   const size_t rb = 8 * (size_t)((p + m + 1) & ~1);
-  AC* parts = reinterpret_cast<AC*>(reinterpret_cast<unsigned char*>(D.ex) + rb);
   const int nparts = dist_kkt_parts(n, R, (size_t)D.cap * sizeof(T) - rb);
-  const int chunk = (R + nparts - 1) / nparts;
-  // column pass: quads of columns over row ranges
-  for (int t = D.rank * NTHREADS + tid; t < nq * nparts; t += D.blocks * NTHREADS) {
-    const int part = t / nq, jq = t - part * nq;
-    const int r0 = part * chunk, r1 = min(R, r0 + chunk);
-    constexpr int RB = sizeof(T) == 4 ? 8 : 4;
-    AC acc[4];
-#pragma unroll 1
-    for (int r = r0; r < r1; r += RB) {
-      T av[RB][4];
-#pragma unroll
-      for (int u = 0; u < RB; ++u)
-        if (r + u < r1) ldg4_row(av[u], rowp(r + u), 4 * jq, n, vec);
-#pragma unroll
-      for (int u = 0; u < RB; ++u)
-        if (r + u < r1) {
-          const V x = xv[r + u];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[c].add(av[u][c], x);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) parts[(size_t)part * 4 * nq + 4 * jq + c] = acc[c];
-  }
-  // row pass: eight lanes per row, two rows per lane group
-  {
-    constexpr int GL = 8, NG = NTHREADS / GL, QB = 4;
-    const int g = tid / GL, gl = tid % GL;
-    for (int r0 = D.rank * 2 * NG; r0 < p + m; r0 += D.blocks * 2 * NG) {
-      const int rr[2] = {r0 + g, r0 + NG + g};
-      const T* rowv[2];
-#pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) rowv[h2] = rowp(n + min(rr[h2], p + m - 1));
-      AC acc[2];
-      for (int qb0 = 0; qb0 < nq; qb0 += GL * QB) {
-        T av[2][QB][4];
-#pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2)
-#pragma unroll
-          for (int u = 0; u < QB; ++u) {
-            const int q = qb0 + gl + u * GL;
-            if (q < nq) ldg4_row(av[h2][u], rowv[h2], 4 * q, n, vec);
-          }
-#pragma unroll
-        for (int u = 0; u < QB; ++u) {
-          const int q = qb0 + gl + u * GL;
-          if (q < nq) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (4 * q + c < n) {
-                const V x = xv[4 * q + c];
-                acc[0].add(av[0][u][c], x);
-                acc[1].add(av[1][u][c], x);
-              }
-          }
-        }
-      }
-#pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {
-#pragma unroll
-        for (int off = GL / 2; off > 0; off >>= 1) acc[h2].shfl_merge(off);
-        if (rr[h2] < p + m && gl == 0) rowres[rr[h2]] = acc[h2];
-      }
-    }
-  }
+  unsigned char* ex = reinterpret_cast<unsigned char*>(D.ex);
+  if (D.blocks == 1 && rb + 32 * (size_t)nq * nparts <= (size_t)D.rest) ex = D.ring + RING_BYTES;
+  AC* rowres = reinterpret_cast<AC*>(ex);
+  AC* parts = reinterpret_cast<AC*>(ex + rb);
+  if (vec && D.ring != nullptr) dist_kkt_passes<true>(D, n, p, m, Q, G, A, xv, rowres, parts, nparts, true);
+  else dist_kkt_passes<false>(D, n, p, m, Q, G, A, xv, rowres, parts, nparts, vec);
   cluster_barrier(D.blocks);
   for (int j = tid; j < n; j += NTHREADS) {
     AC acc;
@@ -1714,6 +1873,13 @@ __device__ __forceinline__ void chol_solve(int p, const T* Mb, int ldM, const T*
   mv_cols(Mb, ldM, p, p, TRI_LOWER, y, scr, [&](int c, T v) { out[c] = v; });
 }
 
+// The same as a routine of its own, for a caller with few registers left.
+template <typename T>
+__device__ __noinline__ void chol_solve_call(int p, const T* Mb, int ldM, const T* rhs, T* y, T* out,
+                                             T* scr) {
+  chol_solve(p, Mb, ldM, rhs, y, out, scr);
+}
+
 // out = M·x with M symmetric, stored as its strict upper triangle in Mb plus diag in dM.
 template <typename T>
 __device__ __forceinline__ void mv_sym_upper(int p, const T* Mb, int ldM, const T* dM,
@@ -1732,15 +1898,6 @@ __device__ __forceinline__ void prefetch_l2(const void* ptr, size_t bytes) {
   const char* c = static_cast<const char*>(ptr);
   for (size_t o = (size_t)threadIdx.x * 128; o < bytes; o += (size_t)NTHREADS * 128)
     asm volatile("prefetch.global.L2 [%0];" :: "l"(c + o));
-}
-
-// Asynchronous 16-byte copy global → shared (cp.async), and the wait for all of a thread's.
-__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(dst_smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(s), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Copies `bytes` bytes from global src to shared dst (both 16-byte aligned) with the whole
@@ -1784,41 +1941,59 @@ namespace qpk {
 // M + D(dsh) into X.  With ws_resident the factors already live in the workspace, and the
 // products are those of Dist when WIDE (the instance may then be shared by the blocks of a
 // cluster, D); otherwise the factors are copied there for the backward pass.
-template <typename T, bool ws_resident, bool WIDE, typename FS, typename FF, typename FV>
+template <typename T, bool ws_resident, int WIDE, typename FS, typename FF, typename FV, typename FB>
 __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& L,
                                          unsigned char* sm, T* SR, T* Mb, int ldMb, T* dM,
-                                         const Dist<T>& D, FS setup, FF factor, FV solve) {
+                                         const Dist<T>& D, FS setup, FF factor, FV solve, FB factors) {
   using V = typename Split<T>::V;
   const int tid = threadIdx.x;
-  const int n = P.n, p = P.p, m = P.m;
-  const int m1 = L.m1, nz = L.nz;
-  T* cb = reinterpret_cast<T*>(sm + L.ocb);
-  double* dv = reinterpret_cast<double*>(sm + L.odbl);
-  double *z = dv, *s = z + n, *lam = s + p, *nu = lam + p;
-  double *rz = nu + m, *rl = rz + n, *rn = rl + p;
-  double *qd = rn + m, *hd = qd + n, *bd = hd + p;   // q, h, b (constant over the solve)
-  V* xs = reinterpret_cast<V*>(sm + L.osplit);
-  T* tv = reinterpret_cast<T*>(sm + L.ovec);
-  const int p4 = (p + 3) / 4 * 4;   // vector strides keep every vector 16-byte aligned
-  T *u = tv, *wv = u + m1, *dzn = wv + m1 + p4, *y = dzn + m1, *dl = y + p4, *dla = dl + p4;
-  T *rhs = dla + p4, *rhsa = rhs + p4, *dsh = rhsa + p4, *mdl = dsh + p4, *tmp = mdl + p4;
-  T *dsv = tmp + p4, *ccv = dsv + p4;
-  float* red = reinterpret_cast<float*>(sm + L.ored);
-  double* dred = reinterpret_cast<double*>(sm + L.ored);
-  Acc<T>* ascr = reinterpret_cast<Acc<T>*>(sm + L.ocb);
-  T* tscr = reinterpret_cast<T*>(sm + L.ocb);
-  const int kscr = (int)(L.cbytes / sizeof(Acc<T>));
-  const int tcap = (int)(L.cbytes / sizeof(T));   // T elements of the work region
-  (void)cb;
+  int n, p, m, m1, nz, p4, kscr, tcap;
+  double *z, *s, *lam, *nu, *rz, *rl, *rn, *qd, *hd, *bd;   // (q, h, b: constant over the solve)
+  V* xs;
+  T *u, *wv, *dzn, *y, *dl, *dla, *rhs, *rhsa, *dsh, *mdl, *tmp, *dsv, *ccv, *tscr;
+  float* red;
+  double* dred;
+  Acc<T>* ascr;
+  const T *Qb, *qb, *Gb, *hb, *Ab, *bb;
+  auto views = [&]() {
+    n = P.n; p = P.p; m = P.m;
+    m1 = L.m1; nz = L.nz;
+    double* dv = reinterpret_cast<double*>(sm + L.odbl);
+    z = dv; s = z + n; lam = s + p; nu = lam + p;
+    rz = nu + m; rl = rz + n; rn = rl + p;
+    qd = rn + m; hd = qd + n; bd = hd + p;
+    xs = reinterpret_cast<V*>(sm + L.osplit);
+    p4 = (p + 3) / 4 * 4;   // vector strides keep every vector 16-byte aligned
+    u = reinterpret_cast<T*>(sm + L.ovec);
+    wv = u + m1; dzn = wv + m1 + p4; y = dzn + m1; dl = y + p4; dla = dl + p4;
+    rhs = dla + p4; rhsa = rhs + p4; dsh = rhsa + p4; mdl = dsh + p4; tmp = mdl + p4;
+    dsv = tmp + p4; ccv = dsv + p4;
+    red = reinterpret_cast<float*>(sm + L.ored);
+    dred = reinterpret_cast<double*>(sm + L.ored);
+    ascr = reinterpret_cast<Acc<T>*>(sm + L.ocb);
+    tscr = reinterpret_cast<T*>(sm + L.ocb);
+    kscr = (int)(L.cbytes / sizeof(Acc<T>));
+    tcap = (int)(L.cbytes / sizeof(T));   // T elements of the work region
+    Qb = P.Q; qb = P.q;
+    Gb = p ? P.G : nullptr; hb = p ? P.h : nullptr;
+    Ab = m ? P.A : nullptr; bb = m ? P.b : nullptr;
+  };
+  auto blocks = [&]() { return WIDE == 2 ? D.blocks : 1; };   // of the cluster
+  views();
+  // After each call of a routine that is not inlined: the sizes and pointers are taken again from
+  // P and L, which a wide size keeps in shared memory, instead of held in registers over the
+  // call.  Held, they and the routines' own registers did not fit in 128 (736 bytes of spill
+  // stores and 2656 of loads, now 148 and 116), and the local memory went to L2, since shared memory
+  // takes the L1 (n = 500, nineq = 20, batch 128: 163M sectors beside 276M of global loads, now 102M).
+  auto renew = [&]() {
+    if constexpr (WIDE != 0) {
+      views();
+      factors(SR, Mb, dM);
+    }
+  };
   __shared__ int s_timeout;
   const unsigned long long t_start = P.time_limit_ns ? globaltimer_ns() : 0ull;
 
-  const T* Qb = P.Q;
-  const T* qb = P.q;
-  const T* Gb = p ? P.G : nullptr;
-  const T* hb = p ? P.h : nullptr;
-  const T* Ab = m ? P.A : nullptr;
-  const T* bb = m ? P.b : nullptr;
   WsLayout W;
   W.init(n, nz, p, m, (int)sizeof(T), ws_resident);
   unsigned char* wsb = P.ws;
@@ -1826,48 +2001,55 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
   T* wX = reinterpret_cast<T*>(wsb + W.oX);
   double* wIt = reinterpret_cast<double*>(wsb + W.oIt);
   int32_t* wSt = reinterpret_cast<int32_t*>(wsb + W.oSt);
-  const int ldS = m1, ldM = ldMb;
 
-  // Products with the factors: wv = [S; RE]·u; with_m(x, out, re): out = M·x (M symmetric, strict
-  // upper triangle plus diag) and, when re, dzn = wv − REᵀx.
+  // Products with the factors: wv = [S; RE]·u; with_m(x, out, mul_m, mul_re): out = M·x (M
+  // symmetric, strict upper triangle plus diag) when mul_m and dzn = wv − REᵀx when mul_re.
   auto with_sr = [&]() {
-    if constexpr (WIDE) {
-      T* o = D.blocks > 1 ? D.ex : wv;
-      dist_rows(D, SR, ldS, m1 + p, m1, false, u, o);
-      cluster_barrier(D.blocks);
-      if (D.blocks > 1) {
-        for (int i = tid; i < m1 + p; i += NTHREADS) wv[i] = o[i];
-        cluster_barrier(D.blocks);
+    if constexpr (WIDE != 0) {
+      dist_rows(D, SR, m1, m1 + p, m1, false, u, blocks() > 1 ? D.ex : wv);
+      renew();
+      cluster_barrier(blocks());
+      if (blocks() > 1) {
+        for (int i = tid; i < m1 + p; i += NTHREADS) wv[i] = D.ex[i];
+        cluster_barrier(blocks());
       }
     } else {
-      if (!mv_rows_xreg<8>(SR, ldS, m1 + p, m1, u, [&](int r, T val) { wv[r] = val; }))
-        mv_rows<8>(SR, ldS, m1 + p, m1, TRI_ALL, u, [&](int r, T val) { wv[r] = val; });
+      if (!mv_rows_xreg<8>(SR, m1, m1 + p, m1, u, [&](int r, T val) { wv[r] = val; }))
+        mv_rows<8>(SR, m1, m1 + p, m1, TRI_ALL, u, [&](int r, T val) { wv[r] = val; });
       __syncthreads();
     }
   };
   auto with_m = [&](const T* x, T* out, bool mul_m, bool mul_re) {
-    if constexpr (WIDE) {
+    if constexpr (WIDE != 0) {
       // exchange buffer: row products | column parts of M | column parts of RE
-      const int npm = dist_col_parts<T>(ldM, p, p), npr = dist_col_parts<T>(ldS, p, m1);
-      T *rowp = D.ex, *mp = rowp + p4, *rp = mp + (size_t)npm * p4;
-      const T* RE = SR + (size_t)m1 * ldS;
+      auto mp = [&]() { return D.ex + p4; };
+      auto rp = [&]() { return mp() + (size_t)dist_col_parts<T>(p, p, p) * p4; };
       if (mul_m) {
-        dist_rows(D, Mb, ldM, p, p, true, x, rowp);
-        dist_cols(D, Mb, ldM, p, p, true, x, mp);
+        dist_rows(D, Mb, p, p, p, true, x, D.ex);
+        renew();
+        dist_cols(D, Mb, p, p, p, true, x, mp());
+        renew();
       }
-      if (mul_re) dist_cols(D, RE, ldS, p, m1, false, x, rp);
-      cluster_barrier(D.blocks);
-      if (mul_m)
+      if (mul_re) {
+        dist_cols(D, SR + (size_t)m1 * m1, m1, p, m1, false, x, rp());
+        renew();
+      }
+      cluster_barrier(blocks());
+      if (mul_m) {
+        const int npm = dist_col_parts<T>(p, p, p);
         for (int i = tid; i < p; i += NTHREADS)
-          out[i] = fma(dM[i], x[i], rowp[i]) + dist_col_sum(mp, p, npm, i);
-      if (mul_re)
-        for (int i = tid; i < m1; i += NTHREADS) dzn[i] = wv[i] - dist_col_sum(rp, m1, npr, i);
-      cluster_barrier(D.blocks);
+          out[i] = fma(dM[i], x[i], D.ex[i]) + dist_col_sum(mp(), p, npm, i);
+      }
+      if (mul_re) {
+        const int npr = dist_col_parts<T>(m1, p, m1);
+        for (int i = tid; i < m1; i += NTHREADS) dzn[i] = wv[i] - dist_col_sum(rp(), m1, npr, i);
+      }
+      cluster_barrier(blocks());
     } else {
       if (mul_re)
-        mv_cols(SR + (size_t)m1 * ldS, ldS, p, m1, TRI_ALL, x, tscr,
+        mv_cols(SR + (size_t)m1 * m1, m1, p, m1, TRI_ALL, x, tscr,
                 [&](int c, T val) { dzn[c] = wv[c] - val; }, tcap);
-      if (mul_m) mv_sym_upper(p, Mb, ldM, dM, x, tmp, out, tscr, tcap);
+      if (mul_m) mv_sym_upper(p, Mb, ldMb, dM, x, tmp, out, tscr, tcap);
     }
   };
   int status = ST_CONV, it = 0, extra = 0, flags = 0;
@@ -1885,7 +2067,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
       xs[i] = Split<T>::make(i < n ? 0.0 : (i < n + p ? lam[i - n] : nu[i - n - p]));
     __syncthreads();
     auto zero = [](int) { return 0.0; };
-    if constexpr (WIDE)
+    if constexpr (WIDE != 0)
     {
       for (int i = tid; i < max(n, p + m); i += NTHREADS) {
         if (i < n) rz[i] = 0.0;
@@ -1893,6 +2075,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
       }
       __syncthreads();
       dist_kkt<T>(D, n, p, m, Qb, Gb, Ab, xs, rz, rl, rn);
+      renew();
     } else
       kkt_apply<T>(n, p, m, Qb, Gb, Ab, xs, ascr, kscr, zero, zero, zero, rz, rl, rn);
     double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1929,7 +2112,8 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     qmx = v[0];
   }
   bool ok = setup(Qb, Ab, Gb, T(0), (T)((sizeof(T) == 4 ? 1e-5f : 1e-12f) * qmx));
-  cluster_barrier(D.blocks);
+  renew();
+  cluster_barrier(blocks());
   if (!ok) {
     float v[4] = {qmx, 0.f, 0.f, 0.f};
     for (int i = tid; i < p + m; i += NTHREADS) {
@@ -1942,7 +2126,8 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     const float scale = fmaxf(fmaxf(v[0], v[1]), 1e-30f);
     delta = (T)((sizeof(T) == 4 ? 1e-4f : 1e-8f) * scale);
     if (isfinite(scale)) ok = setup(Qb, Ab, Gb, delta, T(0));
-    cluster_barrier(D.blocks);
+    renew();
+    cluster_barrier(blocks());
     if (ok) flags |= FLAG_REGQ;
   }
   if (!ok) status = ST_NOTPD;
@@ -1970,7 +2155,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     // Equality-constrained QP: [z; ν] = S·[−q; b], then FP64-residual refinement.
     for (int i = tid; i < m1; i += NTHREADS) u[i] = (i < n) ? -qb[i] : (i < nz ? T(0) : bb[i - nz]);
     __syncthreads();
-    mv_rows<8>(SR, ldS, m1, m1, TRI_ALL, u, [&](int r, T val) {
+    mv_rows<8>(SR, m1, m1, m1, TRI_ALL, u, [&](int r, T val) {
       if (r < n) z[r] = (double)val; else if (r >= nz) nu[r - nz] = (double)val;
     });
     __syncthreads();
@@ -1990,7 +2175,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
       if (v[0] <= 0.01f * tz && v[1] <= 0.01f * tn) break;
       for (int i = tid; i < m1; i += NTHREADS) u[i] = (i < n) ? (T)(-rz[i]) : (i < nz ? T(0) : (T)(-rn[i - nz]));
       __syncthreads();
-      mv_rows<8>(SR, ldS, m1, m1, TRI_ALL, u, [&](int r, T val) {
+      mv_rows<8>(SR, m1, m1, m1, TRI_ALL, u, [&](int r, T val) {
         if (r < n) z[r] += (double)val; else if (r >= nz) nu[r - nz] += (double)val;
       });
       __syncthreads();
@@ -2001,12 +2186,14 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     for (int i = tid; i < m1; i += NTHREADS) u[i] = (i < n) ? -qb[i] : (i < nz ? T(0) : bb[i - nz]);
     __syncthreads();
     ok = factor(dsh);
+    renew();
     if (!ok) status = ST_NOTPD;
     if (ok) {
       with_sr();
       for (int i = tid; i < p; i += NTHREADS) rhs[i] = wv[m1 + i] - hb[i];
       __syncthreads();
       solve(rhs, y, dl, tscr);
+      renew();
       with_m(dl, mdl, false, true);
       float v[4] = {-INFINITY, 0.f, -INFINITY, 0.f};
       for (int i = tid; i < n; i += NTHREADS) z[i] = (double)dzn[i];
@@ -2035,7 +2222,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
       // Residual precision (FP32 factors only): the plain FP32 operator while the previous
       // iteration's μ is above 1e5·mu_tol, the FP64-accurate one from then on.  Convergence
       // is only ever declared on an FP64-accurate residual.
-      bool exact = sizeof(T) == 8 || WIDE;
+      bool exact = sizeof(T) == 8 || WIDE != 0;
       float mu_prev = INFINITY;
       // The KKT residual at the current iterate and its norms (v[0..2]) and μ·p (v[3]).
       auto residual = [&](bool fast, float (&v)[4]) {
@@ -2045,13 +2232,14 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         auto az = [&](int j) { return qd[j]; };
         auto al = [&](int i) { return s[i] - hd[i]; };
         auto an = [&](int i) { return -bd[i]; };
-        if constexpr (WIDE) {
+        if constexpr (WIDE != 0) {
           for (int i = tid; i < n; i += NTHREADS) rz[i] = az(i);
           for (int i = tid; i < p; i += NTHREADS) rl[i] = al(i);
           for (int i = tid; i < m; i += NTHREADS) rn[i] = an(i);
           __syncthreads();
           // always the FP64-accurate form: the matrices' traffic bounds it
           dist_kkt<T>(D, n, p, m, Qb, Gb, Ab, xs, rz, rl, rn);
+          renew();
         } else {
           if (fast) kkt_apply_fast<T>(n, p, m, Qb, Gb, Ab, xs, tscr, tcap, az, al, an, rz, rl, rn);
           else kkt_apply<T>(n, p, m, Qb, Gb, Ab, xs, ascr, kscr, az, al, an, rz, rl, rn);
@@ -2121,12 +2309,12 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         }
         if (P.time_limit_ns) {
           // one block decides for the cluster
-          int* flag = D.blocks > 1 ? reinterpret_cast<int*>(D.ex) : &s_timeout;
+          int* flag = blocks() > 1 ? reinterpret_cast<int*>(D.ex) : &s_timeout;
           if (tid == 0 && D.rank == 0)
             *flag = (globaltimer_ns() - t_start > P.time_limit_ns) ? 1 : 0;
-          cluster_barrier(D.blocks);
+          cluster_barrier(blocks());
           const int out = *flag;
-          cluster_barrier(D.blocks);
+          cluster_barrier(blocks());
           if (out) {
             status = ST_TIMEOUT;
             break;
@@ -2135,7 +2323,9 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         for (int i = tid; i < p; i += NTHREADS) dsh[i] = ratio_to<T>((T)s[i] / (T)lam[i]);
         for (int i = tid; i < m1; i += NTHREADS) u[i] = (i < n) ? (T)(-rz[i]) : (i < nz ? T(0) : (T)(-rn[i - nz]));
         __syncthreads();
-        if (!factor(dsh)) {
+        const bool pd = factor(dsh);
+        renew();
+        if (!pd) {
           status = ST_NOTPD;
           loop_notpd = true;
           break;
@@ -2145,6 +2335,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         for (int i = tid; i < p; i += NTHREADS) rhsa[i] = wv[m1 + i] + (T)(rl[i] - s[i]);
         __syncthreads();
         solve(rhsa, y, dla, tscr);
+        renew();
         with_m(dla, mdl, true, false);
         // Δs from the complementarity row where s ≤ λ and from the primal row
         // GΔz + Δs = −r_λ (with GΔz = RE·u − MΔλ) elsewhere: the first multiplies the
@@ -2179,6 +2370,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         }
         __syncthreads();
         solve(rhs, y, dl, tscr);
+        renew();
         with_m(dl, mdl, true, true);
         float w6[4] = {INFINITY, 0.f, 0.f, 0.f};
         for (int i = tid; i < p; i += NTHREADS) {
@@ -2208,6 +2400,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
         for (int i = tid; i < p; i += NTHREADS) dsh[i] = ratio_to<T>((T)s[i] / (T)lam[i]);
         __syncthreads();
         if (!factor(dsh)) status = ST_NOTPD;
+        renew();
       }
       // Near-degenerate point: some pair with max(λ_i, s_i) ≤ 1e-5·max(1, max_j max(λ_j, s_j)).
       if (status == ST_CONV || status == ST_MAXIT || status == ST_TIMEOUT) {
@@ -2229,6 +2422,11 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
   // An infeasibility certificate is returned scaled to max(‖λ‖∞, ‖ν‖∞) = 1.
   const double dsc = status == ST_INFEAS ? cert_scale : 1.0;
   if (D.rank != 0) return;   // every block holds the same iterate
+  if constexpr (WIDE != 0) {
+    W.init(n, nz, p, m, (int)sizeof(T), ws_resident);
+    wIt = reinterpret_cast<double*>(P.ws + W.oIt);
+    wSt = reinterpret_cast<int32_t*>(P.ws + W.oSt);
+  }
   for (int i = tid; i < n; i += NTHREADS) {
     const double v = bad ? qnan : z[i];
     P.z[i] = (T)v;
@@ -2246,7 +2444,7 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
     wIt[n + 2 * p + i] = v;
   }
   if (!bad && !ws_resident)
-    for (int i = tid; i < p * p; i += NTHREADS) wX[i] = Mb[(size_t)(i / p) * ldM + i % p];
+    for (int i = tid; i < p * p; i += NTHREADS) wX[i] = Mb[(size_t)(i / p) * ldMb + i % p];
   if (tid == 0) {
     wSt[0] = status | flags;
     wSt[1] = STAMP_MAGIC;
@@ -2302,58 +2500,92 @@ __device__ __forceinline__ void fwd_smem_path(const FwdInst<T>& I, unsigned char
   T* cb = reinterpret_cast<T*>(sm + L.ocb);
   const int n = I.n, p = I.p, m = I.m;
   const int tcap = (int)(L.cbytes / sizeof(T));
-  fwd_body<T, false, false>(I, L, sm, SR, Mb, L.ldM, dM, Dist<T>{1, 0, nullptr, 0},
+  fwd_body<T, false, 0>(I, L, sm, SR, Mb, L.ldM, dM, Dist<T>{1, 0, nullptr, 0, nullptr, 0},
       [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
         return sweep_setup<T, SW>(n, p, m, Qb, Ab, Gb, SR, L.ldS, Mb, L.ldM, dM, cb, delta, zthr);
       },
       [&](const T* dsh) { return chol_blk<T, CH, true>(p, Mb, L.ldM, dM, dsh, cb); },
-      [&](const T* rhs, T* y, T* out, T* scr) { chol_solve(p, Mb, L.ldM, rhs, y, out, scr); });
+      [&](const T* rhs, T* y, T* out, T* scr) { chol_solve(p, Mb, L.ldM, rhs, y, out, scr); },
+      [](T*&, T*&, T*&) {});
 }
 
 // One instance on the global-memory path (factors in the workspace, see qp_large.cuh).  TC:
 // whether the setup sweep may take its rank-64 updates on the tensor cores (qp_tc.cuh).  The
-// fixed-size kernel does; the persistent packed kernel does not (its tensor-core variant raised
-// a GPU fault whose cause was not found), so its workspace has no panel-tile region.
-template <typename T, bool TC, bool WIDE>
-__device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned char* sm,
-                                                int blocks, int rank) {
+// fixed-size kernel does; the packed kernels do not (the tensor-core variant of an earlier,
+// persistent one raised a GPU fault whose cause was not found), so their workspaces have no
+// panel-tile region.
+template <typename T>
+struct GlobalPath {   // an instance, its layout and its matrices in the workspace
+  FwdInst<T> I;
   FwdSmem<T> L;
-  L.init(I.n, I.nz, I.p, I.m, true);
-  const int n = I.n, p = I.p, m = I.m, nz = I.nz;
+  Dist<T> D;
+  T *SR, *Mb, *dM, *Aw, *pan, *tcp;
+};
+template <typename T, bool TC>
+__device__ __forceinline__ void init_global_path(GlobalPath<T>& S, const FwdInst<T>& I, unsigned char* sm, int blocks, int rank) {
+  S.I = I;
+  S.L.init(I.n, I.nz, I.p, I.m, true);
   WsLayout W;
-  W.init(n, nz, p, m, (int)sizeof(T), true, TC);
-  T* SR = reinterpret_cast<T*>(I.ws + W.oSR);
-  T* Mb = reinterpret_cast<T*>(I.ws + W.oX);
-  T* dM = reinterpret_cast<T*>(I.ws + W.odM);
-  T* Aw = reinterpret_cast<T*>(I.ws + W.oAw);
-  T* pan = reinterpret_cast<T*>(I.ws + W.oPan);
-  T* cb = reinterpret_cast<T*>(sm + L.ocb);
-  const int tcap = (int)(L.cbytes / sizeof(T));
+  W.init(I.n, I.nz, I.p, I.m, (int)sizeof(T), true, TC);
+  S.SR = reinterpret_cast<T*>(I.ws + W.oSR);
+  S.Mb = reinterpret_cast<T*>(I.ws + W.oX);
+  S.dM = reinterpret_cast<T*>(I.ws + W.odM);
+  S.Aw = reinterpret_cast<T*>(I.ws + W.oAw);
+  S.pan = reinterpret_cast<T*>(I.ws + W.oPan);
+  S.tcp = TC && S.L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr;
   // exchange buffer of the cluster's blocks: the panel scratch, idle outside the factorisations
   // (and in them where the panels are in shared memory)
-  const Dist<T> D{blocks, rank, pan, (int)((W.oTc - W.oPan) / sizeof(T))};
-  fwd_body<T, true, WIDE>(I, L, sm, SR, Mb, p > 0 ? p : 1, dM, D,
+  S.D = Dist<T>{blocks, rank, S.pan, (int)((W.oTc - W.oPan) / sizeof(T)), S.L.ring ? sm + S.L.ocb : nullptr,
+                S.L.ring ? (int)(S.L.cbytes - RING_BYTES) : 0};
+}
+template <typename T, bool TC, int WIDE>
+__device__ __forceinline__ void run_global_path(const GlobalPath<T>& S, unsigned char* sm) {
+  fwd_body<T, true, WIDE>(S.I, S.L, sm, S.SR, S.Mb, S.I.p > 0 ? S.I.p : 1, S.dM, S.D,
       [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
-        return gsweep_setup<T, WIDE>(n, nz, p, m, Qb, Ab, Gb, SR, Mb, dM, pan, L.span_smem != 0, cb,
-                               delta, zthr,
-                               TC && L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr, blocks,
-                               rank);
+        T* cb = reinterpret_cast<T*>(sm + S.L.ocb);
+        if constexpr (WIDE == 2)
+          return gsweep_setup<T, true>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
+                                       S.L.span_smem != 0, cb, delta, zthr, S.tcp, S.D.blocks, S.D.rank);
+        else return gsweep_setup<T, false>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
+                                      S.L.span_smem != 0, cb, delta, zthr, S.tcp, 1, 0);
       },
       [&](const T* dsh) {
         // Small Schur complements: the register-tile routine (M read from and X written to
         // the workspace, panels in shared memory); otherwise the blocked global routine.
-        const int NT = (p + 3) >> 2, nt = NT * (NT + 1) / 2, ldM = p > 0 ? p : 1;
-        if (nt <= NTHREADS) return chol_blk<T, 1, true>(p, Mb, ldM, dM, dsh, cb);
+        const int p = S.I.p, NT = (p + 3) >> 2, nt = NT * (NT + 1) / 2, ldM = p > 0 ? p : 1;
+        T* cb = reinterpret_cast<T*>(sm + S.L.ocb);
+        if (nt <= NTHREADS) return chol_blk<T, 1, true>(p, S.Mb, ldM, S.dM, dsh, cb);
         if constexpr (sizeof(T) == 4) {
-          if (reg_chol_ok(p, 4)) return chol_blk<T, 2, true>(p, Mb, ldM, dM, dsh, cb);
+          if (reg_chol_ok(p, 4)) return chol_blk<T, 2, true>(p, S.Mb, ldM, S.dM, dsh, cb);
         }
-        return gchol_factor<T, WIDE>(p, Mb, dM, dsh, Aw, pan, L.pan_smem != 0, cb, pan, blocks, rank);
+        if constexpr (WIDE == 2)
+          return gchol_factor<T, true>(p, S.Mb, S.dM, dsh, S.Aw, S.pan, S.L.pan_smem != 0, cb, S.pan,
+                                       S.D.blocks, S.D.rank);
+        else return gchol_factor<T, false>(p, S.Mb, S.dM, dsh, S.Aw, S.pan, S.L.pan_smem != 0, cb, S.pan, 1, 0);
       },
       [&](const T* rhs, T* y, T* out, T* scr) {
-        const int ldM = p > 0 ? p : 1;
-        if (reg_chol_ok(p, (int)sizeof(T))) chol_solve(p, Mb, ldM, rhs, y, out, scr);
-        else blk_solve(p, Mb, ldM, rhs, y, out, scr);
-      });
+        const int p = S.I.p, ldM = p > 0 ? p : 1;
+        if (reg_chol_ok(p, (int)sizeof(T))) {
+          if constexpr (WIDE != 0) chol_solve_call(p, S.Mb, ldM, rhs, y, out, scr);
+          else chol_solve(p, S.Mb, ldM, rhs, y, out, scr);
+        }
+        else blk_solve(p, S.Mb, ldM, rhs, y, out, scr);
+      },
+      [&](T*& SR, T*& Mb, T*& dM) { SR = S.SR; Mb = S.Mb; dM = S.dM; });
+}
+template <typename T, bool TC, int WIDE>
+__device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned char* sm,
+                                                int blocks, int rank) {
+  if constexpr (WIDE != 0) {
+    __shared__ GlobalPath<T> S;
+    if (threadIdx.x == 0) init_global_path<T, TC>(S, I, sm, blocks, rank);
+    __syncthreads();
+    run_global_path<T, TC, WIDE>(S, sm);
+  } else {
+    GlobalPath<T> S;
+    init_global_path<T, TC>(S, I, sm, 1, 0);
+    run_global_path<T, TC, 0>(S, sm);
+  }
 }
 
 // Fixed-size batch, shared-memory path: one block per instance.
@@ -2363,16 +2595,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_kernel(const FwdParams<T> 
   fwd_smem_path<T, SW, CH>(fixed_inst(P, blockIdx.x), sm);
 }
 
-// Fixed-size batch, global-memory path: P.blocks blocks (a cluster, where more than one) per
-// instance when WIDE, one otherwise.
-template <typename T, bool WIDE>
+// Fixed-size batch, global-memory path.  WIDE: 0 sizes below the wide line, one block per instance;
+// 1 wide sizes on one block; 2 wide sizes on clusters of P.blocks blocks.  (One block as a kernel of its
+// own: with a run-time number of blocks the setup took 10% longer, n = nineq = 500, batch 128 28.5 ms
+// against 27.8.)
+template <typename T, int WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_large_kernel(const FwdParams<T> P) {
   extern __shared__ __align__(16) unsigned char sm[];
-  if constexpr (WIDE) {
+  if constexpr (WIDE == 2) {
     const int inst = (int)blockIdx.x / P.blocks;
-    fwd_global_path<T, true, true>(fixed_inst(P, inst), sm, P.blocks, (int)blockIdx.x - inst * P.blocks);
+    fwd_global_path<T, true, 2>(fixed_inst(P, inst), sm, P.blocks, (int)blockIdx.x - inst * P.blocks);
   } else {
-    fwd_global_path<T, true, false>(fixed_inst(P, blockIdx.x), sm, 1, 0);
+    fwd_global_path<T, true, WIDE>(fixed_inst(P, blockIdx.x), sm, 1, 0);
   }
 }
 
@@ -2436,16 +2670,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_kernel(const Packed
 // traffic of the factors of 152 instances in flight.  512 uneven instances, forward and
 // backward: 17.4 ms with a persistent kernel of both paths, 16.9 ms now.  The setup sweep runs on CUDA cores (its tensor-core form faulted
 // in an earlier persistent form of this kernel, for a reason that was not found).
-template <typename T, bool WIDE>
+template <typename T, int WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_large_kernel(const PackedFwdParams<T> P) {
   extern __shared__ __align__(16) unsigned char sm[];
-  if constexpr (WIDE) {
+  if constexpr (WIDE == 2) {
     const int k = (int)blockIdx.x / P.blocks;
     const PackedDesc d = P.desc[k];
-    fwd_global_path<T, false, true>(packed_inst(P, d), sm, P.blocks, (int)blockIdx.x - k * P.blocks);
+    fwd_global_path<T, false, 2>(packed_inst(P, d), sm, P.blocks, (int)blockIdx.x - k * P.blocks);
   } else {
     const PackedDesc d = P.desc[blockIdx.x];
-    fwd_global_path<T, false, false>(packed_inst(P, d), sm, 1, 0);
+    fwd_global_path<T, false, WIDE>(packed_inst(P, d), sm, 1, 0);
   }
 }
 

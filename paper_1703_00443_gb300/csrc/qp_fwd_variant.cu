@@ -42,7 +42,8 @@ static cudaError_t launch_clusters(K kernel, const P& params, int count, int blo
 #endif
 template <typename T>
 cudaError_t launch_fwd_large_v(const FwdParams<T>& P, size_t smem, cudaStream_t st) {
-  auto k = P.blocks ? qp_fwd_large_kernel<T, true> : qp_fwd_large_kernel<T, false>;
+  auto k = P.blocks == 0 ? qp_fwd_large_kernel<T, 0>
+                         : (P.blocks == 1 ? qp_fwd_large_kernel<T, 1> : qp_fwd_large_kernel<T, 2>);
   cudaError_t e = prepare_smem(k, smem);
   if (e != cudaSuccess) return e;
 #if !defined(QP_HOST_EMULATION)
@@ -54,7 +55,8 @@ cudaError_t launch_fwd_large_v(const FwdParams<T>& P, size_t smem, cudaStream_t 
 template cudaError_t launch_fwd_large_v<QP_T>(const FwdParams<QP_T>&, size_t, cudaStream_t);
 template <typename T>
 cudaError_t launch_fwd_packed_large_v(const PackedFwdParams<T>& P, size_t smem, cudaStream_t st) {
-  auto k = P.blocks ? qp_fwd_packed_large_kernel<T, true> : qp_fwd_packed_large_kernel<T, false>;
+  auto k = P.blocks == 0 ? qp_fwd_packed_large_kernel<T, 0>
+                         : (P.blocks == 1 ? qp_fwd_packed_large_kernel<T, 1> : qp_fwd_packed_large_kernel<T, 2>);
   cudaError_t e = prepare_smem(k, smem);
   if (e != cudaSuccess) return e;
 #if !defined(QP_HOST_EMULATION)

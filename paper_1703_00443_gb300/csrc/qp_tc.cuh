@@ -184,12 +184,20 @@ __device__ __forceinline__ void cluster_barrier(int blocks) {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   __threadfence();
 }
+// A thread's asynchronous copies (cp_async16) in batches: the end of a batch, and the wait until all
+// batches but the last have arrived.
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_but_one() {
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
 #endif  // __CUDA_ARCH__
 #if !defined(__CUDA_ARCH__)
 __device__ __forceinline__ void cluster_barrier(int blocks) {
   (void)blocks;
   __syncthreads();   // a cluster of one
 }
+__device__ __forceinline__ void cp_async_commit() {}
+__device__ __forceinline__ void cp_async_wait_but_one() {}
 #endif
 
 // Bounded wait for the completion of phase `parity`; false when TC_WAIT_NS ran out.
