@@ -227,7 +227,7 @@ typedef struct qp_packed_sizes {
 /* Host-side planning: dims is a HOST array of B triples (n, nineq, neq).  Fills the HOST
  * arrays desc[B] (in execution order: the sizes->n_global global-path instances first, of
  * them the wide sizes first, then the shared-memory-path ones, each part largest estimated
- * cost first) and *sizes.  The
+ * cost first; of the wide ones, those that several blocks can share first) and *sizes.  The
  * caller copies desc to device memory unchanged and passes it, with sizes, to the packed
  * calls. */
 int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
@@ -240,6 +240,10 @@ int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
 int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* dims,
                       const int8_t* path_hint, const float* cost, qp_instance_desc* desc,
                       qp_packed_sizes* sizes);
+
+/* Host query: how many of a plan's wide instances run on eight, four, two and one block
+ * (counts[0..3]). */
+int qp_packed_blocks(const qp_packed_sizes* sizes, int32_t* counts);
 
 /* Forward pass of a packed batch (device pointers as in qp_forward, packed as above;
  * status/iters/resid indexed by instance id; workspace of sizes->ws_bytes bytes).  The

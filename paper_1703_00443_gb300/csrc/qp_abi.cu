@@ -3,6 +3,8 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
+#include <functional>
 #include <mutex>
 #include <vector>
 
@@ -232,14 +234,66 @@ int blocks_per_instance(int B, bool share) {
 // four blocks each 21.1 ms, at four and two all resident 17.6), and blocks left idle are worth
 // most to the largest (96 requests, 24 shared: at four 15.4 ms, the first ten at eight 13.0).
 struct Levels { int n8, n4, n2; };   // instances at eight, four and two blocks, in this order
-Levels share_levels(int nshare) {
-  const int nsm = num_sms(), most = nsm * 9 / 10;
-  nshare = std::min(nshare, most / 2);
-  int left = most - 2 * nshare;
+int share_most(int nsm) { return nsm * 9 / 10 / 2; }   // instances that have room for two blocks each
+Levels share_levels(int nshare, int nsm) {
+  nshare = std::min(nshare, share_most(nsm));
+  int left = nsm * 9 / 10 - 2 * nshare;
   const int n48 = std::min(nshare, left / 2);
   left -= 2 * n48;
   const int n8 = std::min({n48, left / 4, nsm * 3 / 4 / 8});
   return {n8, n48 - n8, nshare - n48};
+}
+
+// How many of the leading `most` instances of a packed batch to share among several blocks: the number
+// with the least time by a simulation of the block scheduler on `nsm` SMs: none within 2% of that, or
+// else the largest number within 2%.
+// est: the instances' estimated costs in execution order.  An instance's time goes about
+// as the 0.75th power of that estimate (batch 128, (500, 500, 125) against (352, 352, 0) and
+// (400, 200, 50): cost 1 : 0.27 : 0.17, time 1 : 0.37 : 0.29) and as 0.42, 0.55 and 0.72 of the
+// one-block time on eight, four and two blocks.  Sharing a number of instances in between can cost
+// more than sharing none: the blocks of the rest then wait for the clusters (60 instances of n = 500:
+// none shared 25.5 ms, 28 34.5, all 19.1).  Against the best of about 15 measured numbers, for 25 mixes of
+// 16 to 256 instances, the choice was within 1.5% in all but two (9 and 11%); the rule before it (those
+// above 1.2 of the batch's total over all SMs, cut to 28 of 29 to 34) lost 67% on 34 instances of
+// n = 500 (23.0 ms against 13.8) and 16 to 25% on four mixes.
+int share_count(const std::vector<double>& est, int most, int nsm) {
+  const int B = (int)est.size();
+  most = std::min({most, share_most(nsm), 255});
+  if (most <= 0) return 0;
+  std::vector<double> t(B), sum(B + 1, 0.0), heap;
+  for (int i = 0; i < B; ++i) {
+    t[i] = std::pow(std::max(est[i], 0.0), 0.75);
+    sum[i + 1] = sum[i] + t[i];
+  }
+  // an instance within its share of all SMs' time does not set the batch's
+  while (most > 0 && t[most - 1] <= sum[B] / nsm) --most;
+  double best = INFINITY;
+  std::vector<double> T(most + 1, INFINITY);
+  for (int k = most; k >= 0; --k) {
+    const Levels lv = share_levels(k, nsm);
+    const int n4 = lv.n8 + lv.n4;
+    double longest = 0.0;
+    for (int i = 0; i < k; ++i)
+      longest = std::max(longest, t[i] * (i < lv.n8 ? 0.42 : i < n4 ? 0.55 : 0.72));
+    if (longest > 1.02 * best || (k < B && t[k] > 1.02 * best)) continue;
+    // the rest go, in order, to the SM that is free first
+    heap.assign(std::max(nsm - (8 * lv.n8 + 4 * lv.n4 + 2 * lv.n2), 0), 0.0);
+    for (int i = 0; i < k; ++i)
+      heap.insert(heap.end(), i < lv.n8 ? 8 : i < n4 ? 4 : 2,
+                  t[i] * (i < lv.n8 ? 0.42 : i < n4 ? 0.55 : 0.72));
+    std::make_heap(heap.begin(), heap.end(), std::greater<double>());
+    for (int i = k; i < B && longest <= 1.02 * best; ++i) {
+      std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
+      heap.back() += t[i];
+      longest = std::max(longest, heap.back());
+      std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+    }
+    T[k] = longest;
+    best = std::min(best, longest);
+  }
+  for (int k = most; k > 0 && T[0] > 1.02 * best; --k)
+    if (T[k] <= 1.02 * best) return k;
+  return 0;
 }
 
 namespace qpk {
@@ -402,7 +456,8 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   int64_t ows = 256;   // first 256 bytes: the two work-queue counters
   int sw_need = 1, ch_need = 1;
   size_t fsm = 0, bsm = 0;
-  int nwide = 0, nshare = 0;
+  int nwide = 0, nable = 0;   // wide instances, and those of them that several blocks can share
+  std::vector<char> cls(B);   // execution order of the classes, last first
   std::vector<std::pair<double, int>> order;
   for (int i = 0; i < B; ++i) {
     const int n = dims[3 * i], p = dims[3 * i + 1], m = dims[3 * i + 2];
@@ -414,6 +469,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     qp_instance_desc& d = desc[i];
     d.n = n; d.nineq = p; d.neq = m; d.id = i; d.nz = pl.nz;
     d.flags = (pl.large ? 1 : 0) | (pl.wide ? 2 : 0);
+    cls[i] = (char)(d.flags + (pl.share ? 1 : 0));
     d.oQ = oQ; d.oq = oq; d.oG = oG; d.oh = oh; d.oA = oA; d.ob = ob;
     d.oz = oq; d.olam = oh; d.onu = ob; d.ows = ows;
     // Offsets padded to multiples of 4 elements keep every instance's rows 16-byte aligned.
@@ -427,6 +483,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     } else {
       ++S.n_global;
       if (pl.wide) ++nwide;
+      if (pl.share) ++nable;
     }
     fsm = std::max(fsm, pl.fsmem);
     bsm = std::max(bsm, pl.bsmem);
@@ -439,13 +496,13 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     for (int k = 0; k < 3; ++k)
       if (sws[k] >= sw_need && qpk::fwd_variant_exists(esz, sws[k], c)) { sw = sws[k]; ch = c; break; }
   if (!sw) return QP_EUNSUPPORTED;
-  // Execution order: the global-path instances of wide sizes first, then the other global-path
-  // ones, then the shared-memory-path ones (separate kernels), each part largest estimated cost
-  // first (longest-processing-time).
+  // Execution order: the global-path instances of wide sizes first (those that several blocks can
+  // share before the others), then the other global-path ones, then the shared-memory-path ones
+  // (separate kernels), each part largest estimated cost first (longest-processing-time).
   std::vector<qp_instance_desc> tmp(desc, desc + B);
   std::stable_sort(order.begin(), order.end(),
                    [&](const std::pair<double, int>& x, const std::pair<double, int>& y) {
-                     const int gx = tmp[x.second].flags & 3, gy = tmp[y.second].flags & 3;
+                     const int gx = cls[x.second], gy = cls[y.second];
                      return gx != gy ? gx > gy : x.first > y.first;
                    });
   for (int k = 0; k < B; ++k) desc[k] = tmp[order[k].second];
@@ -454,24 +511,21 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   S.ws_bytes = ows;
   S.fwd_smem = (int64_t)fsm; S.bwd_smem = (int64_t)bsm;
   S.sw = sw; S.ch = ch;
-  // Wide instances to share among several blocks: leading ones (largest first) whose own
-  // estimated time on one SM would exceed 1.2 of the batch's total over all SMs, and so set
-  // the batch's time: sharing more of them only takes SMs from whole instances, which use them
-  // better.  Where four blocks each would hold nearly all SMs, the last few stay on one, so
-  // that six have eight: they would wait for the first otherwise (128 requests: 33 shared
-  // 15.7 ms, 28 shared 13.3).  The plan keeps both counts in `reserved`.
-  double total = 0.0;
-  for (const auto& x : order) total += x.first;
-  const double limit = 1.2 * total / num_sms();
-  const int budget = num_sms() * 9 / 10;
-  while (nshare < std::min({nwide, 255, budget / 2}) && order[nshare].first > limit) {
-    const qp_instance_desc& d = desc[nshare];
-    if (!panels_in_smem(dtype, d.n, d.nz, d.nineq, d.neq)) break;
-    ++nshare;
-  }
-  if (4 * nshare <= budget) nshare = std::min(nshare, std::max(budget / 4 - 6, 0));
+  // The plan keeps the number of wide instances and how many of them several blocks share.
+  std::vector<double> est;
+  for (const auto& x : order) est.push_back(x.first);
+  const int nshare = share_count(est, nable, num_sms());
   S.reserved = nwide << 8 | nshare;
   *sizes = S;
+  return QP_OK;
+}
+
+int qp_packed_blocks(const qp_packed_sizes* sizes, int32_t* counts) {
+  if (!sizes || !counts) return QP_EINVAL;
+  const int nwide = std::max(sizes->reserved >> 8, 0);
+  const Levels lv = share_levels(std::min(sizes->reserved & 255, nwide), num_sms());
+  counts[0] = lv.n8; counts[1] = lv.n4; counts[2] = lv.n2;
+  counts[3] = nwide - lv.n8 - lv.n4 - lv.n2;
   return QP_OK;
 }
 
@@ -534,7 +588,7 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
 #if defined(QP_HOST_EMULATION)
   const Levels lv{0, 0, 0};   // the host emulation runs one block at a time
 #else
-  const Levels lv = share_levels(nshare);
+  const Levels lv = share_levels(nshare, nsm);
 #endif
   int off = 0;
   auto add = [&](int kind, int cnt) {

@@ -1,0 +1,39 @@
+"""The plan's choice of the wide instances that several blocks share (host logic, no GPU needed; the
+counts hold for 152 SMs, which the planner takes where no device is visible)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_1703_00443_gb300 import _lib
+
+
+def _plan(sizes, cost=None):
+    """(execution order, instances on 8, 4, 2 and 1 blocks) of a packed plan."""
+    lib = _lib.load()
+    B = len(sizes)
+    dims = np.ascontiguousarray(np.array(sizes, dtype=np.int32))
+    desc, S, o = (_lib.QPInstanceDesc * B)(), _lib.QPPackedSizes(), _lib.QPOptions()
+    lib.qp_default_options(0, ctypes.byref(o))
+    c = None if cost is None else np.ascontiguousarray(cost, dtype=np.float32)
+    assert lib.qp_packed_plan_ex(ctypes.byref(o), 0, B, dims.ctypes.data_as(ctypes.c_void_p), None,
+                                 None if c is None else c.ctypes.data_as(ctypes.c_void_p), desc,
+                                 ctypes.byref(S)) == 0
+    counts = (ctypes.c_int32 * 4)()
+    assert lib.qp_packed_blocks(ctypes.byref(S), counts) == 0
+    return [desc[k].id for k in range(B)], list(counts)
+
+
+@pytest.mark.parametrize("count", [1, 14, 18, 28, 29, 30, 33, 34, 35, 36, 60, 68])
+def test_equal_large_instances_are_all_shared(count):
+    """One left on a single block would take twice as long as the others (34 of n = 500, 28 of them
+    shared: 23 ms against 14)."""
+    _, (n8, n4, n2, n1) = _plan([(500, 500, 125)] * count)
+    assert n8 + n4 + n2 == count and n1 == 0
+    assert 8 * n8 + 4 * n4 + 2 * n2 <= 152 * 9 // 10
+
+
+def test_more_equal_instances_than_pairs_of_sms_are_not_shared():
+    """69 clusters of two would not be resident at once; the rest would wait for them."""
+    for count in (100, 152, 400):
+        assert _plan([(500, 500, 125)] * count)[1] == [0, 0, 0, count]
