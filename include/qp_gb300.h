@@ -236,7 +236,8 @@ int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
 /* qp_packed_plan with per-instance hints from a tuner: path_hint[i] (may be NULL) is 0 for
  * the automatic choice, 1 for the global-memory kernel, 2 for the shared-memory kernel
  * (QP_EUNSUPPORTED if it cannot take that size); cost[i] (may be NULL) replaces the built-in
- * cost estimate that orders the instances (largest first). */
+ * cost estimate that orders the instances (largest first).  Any scale will do: which instances
+ * several blocks share follows from the built-in estimate. */
 int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* dims,
                       const int8_t* path_hint, const float* cost, qp_instance_desc* desc,
                       qp_packed_sizes* sizes);

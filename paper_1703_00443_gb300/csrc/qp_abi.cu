@@ -202,8 +202,8 @@ int num_sms() {
 }
 
 // Rough relative cost of one instance (FMA counts of the setup sweep, ~12 interior point
-// iterations and the backward solve; the global path runs about 3× slower per FMA); used
-// only to order the work queue largest first.
+// iterations and the backward solve; the global path runs about 3× slower per FMA): the
+// instances' order, largest first, and the choice of those that several blocks share.
 double est_cost(int n, int nz, int p, int m, bool large) {
   const double m1 = nz + m, N = m1 + p;
   const double c = m1 * N * N + 12.0 * (p * (double)p * p / 3.0 + 2.0 * n * N) + N * N;
@@ -458,6 +458,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   size_t fsm = 0, bsm = 0;
   int nwide = 0, nable = 0;   // wide instances, and those of them that several blocks can share
   std::vector<char> cls(B);   // execution order of the classes, last first
+  std::vector<double> own(B);   // the planner's own cost estimates
   std::vector<std::pair<double, int>> order;
   for (int i = 0; i < B; ++i) {
     const int n = dims[3 * i], p = dims[3 * i + 1], m = dims[3 * i + 2];
@@ -487,7 +488,8 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
     }
     fsm = std::max(fsm, pl.fsmem);
     bsm = std::max(bsm, pl.bsmem);
-    order.push_back({cost ? (double)cost[i] : est_cost(n, pl.nz, p, m, pl.large), i});
+    own[i] = est_cost(n, pl.nz, p, m, pl.large);
+    order.push_back({cost ? (double)cost[i] : own[i], i});
   }
   // Register-tile variant covering every shared-memory-path instance.
   int sw = 0, ch = 0;
@@ -511,9 +513,10 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   S.ws_bytes = ows;
   S.fwd_smem = (int64_t)fsm; S.bwd_smem = (int64_t)bsm;
   S.sw = sw; S.ch = ch;
-  // The plan keeps the number of wide instances and how many of them several blocks share.
+  // The plan keeps the number of wide instances and how many of them several blocks share (by the
+  // planner's own estimates: a caller's costs may be ranks, or no times at all).
   std::vector<double> est;
-  for (const auto& x : order) est.push_back(x.first);
+  for (const auto& x : order) est.push_back(own[x.second]);
   const int nshare = share_count(est, nable, num_sms());
   S.reserved = nwide << 8 | nshare;
   *sizes = S;

@@ -37,3 +37,14 @@ def test_more_equal_instances_than_pairs_of_sms_are_not_shared():
     """69 clusters of two would not be resident at once; the rest would wait for them."""
     for count in (100, 152, 400):
         assert _plan([(500, 500, 125)] * count)[1] == [0, 0, 0, count]
+
+
+@pytest.mark.parametrize("cost", [[0.0] * 5, [1.0, 2.0, 3.0, 4.0, 5.0], [1e-3] * 4 + [9e-3],
+                                  [float("inf")] * 5])
+def test_costs_order_the_instances_and_do_not_choose_the_shared_ones(cost):
+    """Costs that are all equal, ranks, or no times at all: the four large instances are shared, in the
+    order of the costs; the fifth is not worth it and cannot be (the panels of 600 inequalities are in
+    global memory), so it comes after them."""
+    order, counts = _plan([(512, 512, 128)] * 4 + [(352, 600, 0)], cost)
+    assert order == (sorted(range(4), key=lambda i: -cost[i]) + [4])
+    assert counts == [4, 0, 0, 1]
