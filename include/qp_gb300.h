@@ -218,7 +218,9 @@ typedef struct qp_packed_sizes {
   int64_t nz, nlam, nnu;            /* elements of each packed output                   */
   int64_t ws_bytes;                 /* workspace bytes, 256-byte aligned                */
   int64_t fwd_smem, bwd_smem;       /* dynamic shared memory of the packed kernels      */
-  int32_t sw, ch;                   /* register-tile variant of the shared-memory path  */
+  int32_t sw, ch;                   /* register-tile variant of the shared-memory path; bits
+                                       8 and up of ch: SMs that the shared instances may
+                                       take, 0 for all                                  */
   int32_t n_global;                 /* instances on the global-memory path              */
   int32_t reserved;          /* wide instances << 8 | those shared by several blocks; 0:
                                 every global-path instance runs on one block            */
@@ -241,6 +243,14 @@ int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
 int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* dims,
                       const int8_t* path_hint, const float* cost, qp_instance_desc* desc,
                       qp_packed_sizes* sizes);
+
+/* qp_packed_plan_ex for a batch that has the device to itself only in part: its shared instances take
+ * at most `sms` SMs (0: none is shared; negative: all SMs, as the calls above plan).  A batch planned
+ * for all SMs beside other batches is no faster and holds up the others: n = 500 takes 10 ms on
+ * eight SMs against 22 on one.  The results do not depend on it. */
+int qp_packed_plan_sms(const qp_options* opt, int dtype, int B, const int32_t* dims,
+                       const int8_t* path_hint, const float* cost, int sms, qp_instance_desc* desc,
+                       qp_packed_sizes* sizes);
 
 /* Host query: how many of a plan's wide instances run on eight, four, two and one block
  * (counts[0..3]). */

@@ -138,6 +138,9 @@ EXPORTS = {
     "qp_packed_plan_ex": (c_int, [ctypes.POINTER(QPOptions), c_int, c_int, c_void_p, c_void_p,
                                   c_void_p, ctypes.POINTER(QPInstanceDesc),
                                   ctypes.POINTER(QPPackedSizes)]),
+    "qp_packed_plan_sms": (c_int, [ctypes.POINTER(QPOptions), c_int, c_int, c_void_p, c_void_p,
+                                   c_void_p, c_int, ctypes.POINTER(QPInstanceDesc),
+                                   ctypes.POINTER(QPPackedSizes)]),
     "qp_packed_blocks": (c_int, [ctypes.POINTER(QPPackedSizes), c_void_p]),
     "qp_forward_packed": (c_int, [ctypes.POINTER(QPOptions), c_int, c_int, c_void_p,
                                   ctypes.POINTER(QPPackedSizes)] + [c_void_p] * 13 + [c_size_t, c_void_p]),

@@ -149,10 +149,13 @@ static_assert(sizeof(qp_instance_desc) == sizeof(qpk::PackedDesc), "descriptor l
 // Non-blocking side streams with their fork/join events, created on first use (host-side
 // resources, not device memory) and kept for the life of the process.  A caller's stream
 // gets its own set (up to kSideSlots per device; beyond that, streams share sets by
-// hash), so packed calls issued on different streams do not queue behind one another.
+// hash), so packed calls issued on different streams do not queue behind one another.  A set has as
+// many streams as its calls have needed: with five in each, 16 callers would have 96 streams,
+// more than the hardware's connections.
 struct SideStream {
   cudaStream_t owner = nullptr;   // the caller stream this slot serves
   bool used = false;
+  int count = 0;                  // streams created
   cudaStream_t s[5] = {};
   cudaEvent_t fork = nullptr, join[5] = {};
   std::mutex mu;
@@ -175,21 +178,29 @@ SideStream* side_stream(cudaStream_t owner) {
   for (int i = 0; i < kSideSlots && !x; ++i)
     if (!row[i].used) x = &row[i];
   if (!x) x = &row[(reinterpret_cast<uintptr_t>(owner) >> 4) % kSideSlots];
-  if (!x->used) {
-    bool ok = x->fork || cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < 5; ++i) {
-      ok = ok && (x->s[i] || cudaStreamCreateWithFlags(&x->s[i], cudaStreamNonBlocking) == cudaSuccess);
-      ok = ok && (x->join[i] ||
-                  cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess);
-    }
-    if (!ok) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    x->used = true;
-    x->owner = owner;
-  }
+  x->used = true;
+  x->owner = owner;
   return x;
+}
+
+// The set's streams, at least `want` of them if they are to be had (the set's mutex is held);
+// returns how many there are.
+int side_streams(SideStream* x, int want) {
+  if (!x->fork && cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  while (x->count < want) {
+    const int i = x->count;
+    if ((!x->s[i] && cudaStreamCreateWithFlags(&x->s[i], cudaStreamNonBlocking) != cudaSuccess) ||
+        (!x->join[i] &&
+         cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) != cudaSuccess)) {
+      cudaGetLastError();
+      break;
+    }
+    ++x->count;
+  }
+  return x->count;
 }
 
 int num_sms() {
@@ -242,6 +253,12 @@ Levels share_levels(int nshare, int nsm) {
   left -= 2 * n48;
   const int n8 = std::min({n48, left / 4, nsm * 3 / 4 / 8});
   return {n8, n48 - n8, nshare - n48};
+}
+
+// The SMs that a plan's shared instances may take: those of the device, or what the plan was given.
+int share_sms(const qp_packed_sizes* sizes, int nsm) {
+  const int sms = sizes->ch >> 8;
+  return sms > 0 ? std::min(sms, nsm) : nsm;
 }
 
 // How many of the leading `most` instances of a packed batch to share among several blocks: the number
@@ -446,6 +463,12 @@ int qp_packed_plan(const qp_options* opt, int dtype, int B, const int32_t* dims,
 int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* dims,
                       const int8_t* path_hint, const float* cost, qp_instance_desc* desc,
                       qp_packed_sizes* sizes) {
+  return qp_packed_plan_sms(opt, dtype, B, dims, path_hint, cost, -1, desc, sizes);
+}
+
+int qp_packed_plan_sms(const qp_options* opt, int dtype, int B, const int32_t* dims,
+                       const int8_t* path_hint, const float* cost, int sms, qp_instance_desc* desc,
+                       qp_packed_sizes* sizes) {
   if ((dtype != QP_F32 && dtype != QP_F64) || B < 0 || !sizes || (B > 0 && (!dims || !desc)))
     return QP_EINVAL;
   qp_options o;
@@ -517,7 +540,10 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
   // planner's own estimates: a caller's costs may be ranks, or no times at all).
   std::vector<double> est;
   for (const auto& x : order) est.push_back(own[x.second]);
-  const int nshare = share_count(est, nable, num_sms());
+  const int nsm = num_sms();
+  if (sms < 0 || sms > nsm) sms = nsm;
+  const int nshare = share_count(est, nable, sms);
+  if (nshare > 0 && sms < nsm) S.ch |= sms << 8;
   S.reserved = nwide << 8 | nshare;
   *sizes = S;
   return QP_OK;
@@ -526,7 +552,7 @@ int qp_packed_plan_ex(const qp_options* opt, int dtype, int B, const int32_t* di
 int qp_packed_blocks(const qp_packed_sizes* sizes, int32_t* counts) {
   if (!sizes || !counts) return QP_EINVAL;
   const int nwide = std::max(sizes->reserved >> 8, 0);
-  const Levels lv = share_levels(std::min(sizes->reserved & 255, nwide), num_sms());
+  const Levels lv = share_levels(std::min(sizes->reserved & 255, nwide), share_sms(sizes, num_sms()));
   counts[0] = lv.n8; counts[1] = lv.n4; counts[2] = lv.n2;
   counts[3] = nwide - lv.n8 - lv.n4 - lv.n2;
   return QP_OK;
@@ -564,7 +590,7 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
                                     (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns,
                                     kind};
       return kind >= 0 ? qpk::launch_fwd_packed_large_f32(P, (size_t)sizes->fwd_smem, s)
-                  : qpk::launch_fwd_packed_f32(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem,
+                  : qpk::launch_fwd_packed_f32(P, sizes->sw, sizes->ch & 255, (size_t)sizes->fwd_smem,
                                                grid, s);
     }
     qpk::PackedFwdParams<double> P{cnt, (const qpk::PackedDesc*)desc + off, (int*)workspace,
@@ -574,7 +600,7 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
                                    (unsigned char*)workspace, o.tol, o.mu_tol, o.max_iter, tl_ns,
                                    kind};
     return kind >= 0 ? qpk::launch_fwd_packed_large_f64(P, (size_t)sizes->fwd_smem, s)
-                : qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch, (size_t)sizes->fwd_smem,
+                : qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch & 255, (size_t)sizes->fwd_smem,
                                              grid, s);
   };
   // Up to six kernels side by side: the largest wide instances with eight, four and two blocks
@@ -591,7 +617,7 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
 #if defined(QP_HOST_EMULATION)
   const Levels lv{0, 0, 0};   // the host emulation runs one block at a time
 #else
-  const Levels lv = share_levels(nshare, nsm);
+  const Levels lv = share_levels(nshare, share_sms(sizes, nsm));
 #endif
   int off = 0;
   auto add = [&](int kind, int cnt) {
@@ -609,25 +635,26 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
     return e == cudaSuccess ? QP_OK : QP_ECUDA;
   }
   SideStream* ss = side_stream(st);
+  bool ok = true;
   if (!ss) {   // no side streams to be had: one after the other
-    bool ok = true;
     for (int i = 0; i < np; ++i)
       ok = launch(parts[i].kind, parts[i].off, parts[i].cnt, st) == cudaSuccess && ok;
     return ok ? QP_OK : QP_ECUDA;
   }
   std::lock_guard<std::mutex> lk(ss->mu);
-  if (cudaEventRecord(ss->fork, st) != cudaSuccess) return QP_ECUDA;
+  const int side = std::min(side_streams(ss, np - 1), np - 1);   // fewer: some queue behind others
+  if (side > 0 && cudaEventRecord(ss->fork, st) != cudaSuccess) return QP_ECUDA;
   if (launch(parts[0].kind, parts[0].off, parts[0].cnt, st) != cudaSuccess) return QP_ECUDA;
-  bool ok = true;
-  for (int i = 1; i < np; ++i) {
-    cudaStream_t s = ss->s[i - 1];
-    if (cudaStreamWaitEvent(s, ss->fork, 0) != cudaSuccess) return QP_ECUDA;
-    ok = launch(parts[i].kind, parts[i].off, parts[i].cnt, s) == cudaSuccess && ok;
-    // joined whether or not the launch succeeded
-    if (cudaEventRecord(ss->join[i - 1], s) != cudaSuccess ||
-        cudaStreamWaitEvent(st, ss->join[i - 1], 0) != cudaSuccess)
+  for (int k = 0; k < side; ++k)
+    if (cudaStreamWaitEvent(ss->s[k], ss->fork, 0) != cudaSuccess) return QP_ECUDA;
+  for (int i = 1; i < np; ++i)
+    ok = launch(parts[i].kind, parts[i].off, parts[i].cnt, side > 0 ? ss->s[(i - 1) % side] : st) ==
+             cudaSuccess && ok;
+  // joined whether or not the launches succeeded
+  for (int k = 0; k < side; ++k)
+    if (cudaEventRecord(ss->join[k], ss->s[k]) != cudaSuccess ||
+        cudaStreamWaitEvent(st, ss->join[k], 0) != cudaSuccess)
       return QP_ECUDA;
-  }
   return ok ? QP_OK : QP_ECUDA;
 }
 

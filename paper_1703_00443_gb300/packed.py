@@ -32,11 +32,13 @@ class PackedForward:
 
 class PackedBatch:
     """Plan, workspace and descriptors of one batch composition (reusable across calls and
-    safe to capture in a CUDA graph once built)."""
+    safe to capture in a CUDA graph once built).  ``sms``: SMs that its shared instances may take where
+    other work runs beside it (default: all; results do not depend on it)."""
 
     KEYS = ("Q", "q", "G", "h", "A", "b")
 
-    def __init__(self, dims, dtype=torch.float32, device="cuda", options=None, tuning=None):
+    def __init__(self, dims, dtype=torch.float32, device="cuda", options=None, tuning=None,
+                 sms=-1):
         self.dims = np.ascontiguousarray(np.asarray(dims, dtype=np.int32).reshape(-1, 3))
         self.B = self.dims.shape[0]
         self.dtype = dtype
@@ -50,11 +52,11 @@ class PackedBatch:
         if tuning is not None:
             # per-instance kernel path and predicted time from a measured tuning table
             hints, cost = tuning.plan_arrays(self.dims)
-        rc = lib.qp_packed_plan_ex(ctypes.byref(self.options), self.code, self.B,
-                                   self.dims.ctypes.data_as(ctypes.c_void_p),
-                                   None if hints is None else hints.ctypes.data_as(ctypes.c_void_p),
-                                   None if cost is None else cost.ctypes.data_as(ctypes.c_void_p),
-                                   self.desc_host, ctypes.byref(self.sizes))
+        rc = lib.qp_packed_plan_sms(ctypes.byref(self.options), self.code, self.B,
+                                    self.dims.ctypes.data_as(ctypes.c_void_p),
+                                    None if hints is None else hints.ctypes.data_as(ctypes.c_void_p),
+                                    None if cost is None else cost.ctypes.data_as(ctypes.c_void_p),
+                                    sms, self.desc_host, ctypes.byref(self.sizes))
         _check(rc)
         raw = bytes(memoryview(self.desc_host))[: self.B * ctypes.sizeof(_lib.QPInstanceDesc)]
         self.desc = torch.frombuffer(bytearray(raw), dtype=torch.uint8).to(self.device) \
