@@ -2544,10 +2544,11 @@ __device__ __forceinline__ void run_global_path(const GlobalPath<T>& S, unsigned
       [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
         T* cb = reinterpret_cast<T*>(sm + S.L.ocb);
         if constexpr (WIDE == 2)
-          return gsweep_setup<T, true>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
+          return gsweep_setup<T, true, TC>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
                                        S.L.span_smem != 0, cb, delta, zthr, S.tcp, S.D.blocks, S.D.rank);
-        else return gsweep_setup<T, false>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
-                                      S.L.span_smem != 0, cb, delta, zthr, S.tcp, 1, 0);
+        else
+          return gsweep_setup<T, false, TC>(S.I.n, S.I.nz, S.I.p, S.I.m, Qb, Ab, Gb, S.SR, S.Mb, S.dM, S.pan,
+                                            S.L.span_smem != 0, cb, delta, zthr, S.tcp, 1, 0);
       },
       [&](const T* dsh) {
         // Small Schur complements: the register-tile routine (M read from and X written to
@@ -2561,7 +2562,8 @@ __device__ __forceinline__ void run_global_path(const GlobalPath<T>& S, unsigned
         if constexpr (WIDE == 2)
           return gchol_factor<T, true>(p, S.Mb, S.dM, dsh, S.Aw, S.pan, S.L.pan_smem != 0, cb, S.pan,
                                        S.D.blocks, S.D.rank);
-        else return gchol_factor<T, false>(p, S.Mb, S.dM, dsh, S.Aw, S.pan, S.L.pan_smem != 0, cb, S.pan, 1, 0);
+        else
+          return gchol_factor<T, false>(p, S.Mb, S.dM, dsh, S.Aw, S.pan, S.L.pan_smem != 0, cb, S.pan, 1, 0);
       },
       [&](const T* rhs, T* y, T* out, T* scr) {
         const int p = S.I.p, ldM = p > 0 ? p : 1;

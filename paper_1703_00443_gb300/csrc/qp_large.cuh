@@ -35,7 +35,8 @@ __host__ __device__ inline int round4(int x) { return (x + 3) & ~3; }
 // negated where the swept matrix holds −S and −M, so SR = [S; RE] and Mb/dM hold M exactly
 // as the register-tile sweep leaves them.
 // WIDE: the work is dealt to the `blocks` blocks of a cluster, of which this is block `rank`.
-template <typename T, bool WIDE>
+// TC: whether the tensor-core routine is compiled in (tcp: its panel tiles, or null).
+template <typename T, bool WIDE, bool TC>
 __device__ __noinline__ bool gsweep_setup(int n, int nz, int p, int m, const T* __restrict__ Q,
                                           const T* __restrict__ A, const T* __restrict__ G,
                                           T* SR, T* Mb, T* dM, T* pan, bool pan_in_sm, T* sm,
@@ -68,7 +69,7 @@ __device__ __noinline__ bool gsweep_setup(int n, int nz, int p, int m, const T* 
   const int RTp = (p + 7) >> 3, CTp = (p + 3) >> 2;    // tile rows / columns of the λλ block
   int kstart = 0;
 #if defined(__CUDA_ARCH__) || defined(QP_HOST_EMULATION)
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4 && TC) {
     // FP32 with the workspace's panel tiles: every pivot in 64-pivot superblocks on the
     // tensor cores (the last one partial), none left for the 16-pivot blocks below.  Not for
     // the regularised retry of a singular Q (delta > 0): its Schur complements are

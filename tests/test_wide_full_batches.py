@@ -26,6 +26,17 @@ def test_wide_kernels_hold_no_spilled_views_over_their_calls():
     assert found and all(int(loads) <= 2656 // 4 for _, loads in found), found
 
 
+def test_packed_kernels_carry_no_tensor_core_routine():
+    """They never call it (by the compiler's report, kept by the build)."""
+    log = os.path.join(_lib.BUILD, "fwd_f32_large.ptxas.log")
+    if not os.path.exists(log):
+        pytest.skip("the library was not built here")
+    kernels = open(log).read().split("Compiling entry function")[1:]
+    packed = [k for k in kernels if "qp_fwd_packed_large_kernel" in k.split("\n")[0]]
+    assert len(packed) == 3 and not any("tc_sweep_superblocks" in k for k in packed)
+    assert sum("tc_sweep_superblocks" in k for k in kernels) == 3      # the fixed-size ones do
+
+
 # rows of one lane group and one more, two rows per group with a partial batch, rows off 16-byte
 # boundaries, FP64 (a quad is two copies) with and without equalities
 @pytest.mark.gpu
