@@ -2152,7 +2152,10 @@ __device__ __forceinline__ void fwd_body(const FwdInst<T>& P, const FwdSmem<T>& 
   }
 
   if (ok && p == 0) {
-    // Equality-constrained QP: [z; ν] = S·[−q; b], then FP64-residual refinement.
+    // Equality-constrained QP: [z; ν] = S·[−q; b], then FP64-residual refinement.  By the first block
+    // of a cluster alone: the products are a fraction of the setup, which the others shared, and nothing
+    // below waits for them.
+    if (WIDE == 2 && D.rank != 0) return;
     for (int i = tid; i < m1; i += NTHREADS) u[i] = (i < n) ? -qb[i] : (i < nz ? T(0) : bb[i - nz]);
     __syncthreads();
     mv_rows<8>(SR, m1, m1, m1, TRI_ALL, u, [&](int r, T val) {
