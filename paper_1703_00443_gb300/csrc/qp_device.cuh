@@ -2558,6 +2558,22 @@ __device__ __forceinline__ void run_global_path(const GlobalPath<T>& S, unsigned
         // the workspace, panels in shared memory); otherwise the blocked global routine.
         const int p = S.I.p, NT = (p + 3) >> 2, nt = NT * (NT + 1) / 2, ldM = p > 0 ? p : 1;
         T* cb = reinterpret_cast<T*>(sm + S.L.ocb);
+        if (WIDE == 2 && reg_chol_ok(p, (int)sizeof(T))) {
+          // by the first block of the cluster alone (one chain of dependent steps whoever takes it); its
+          // answer goes through the Cholesky's work matrix, which these sizes leave idle
+          int* pd = reinterpret_cast<int*>(S.Aw);
+          if (S.D.rank == 0) {
+            bool ok;
+            if constexpr (sizeof(T) == 4)
+              ok = nt <= NTHREADS ? chol_blk<T, 1, true>(p, S.Mb, ldM, S.dM, dsh, cb)
+                                  : chol_blk<T, 2, true>(p, S.Mb, ldM, S.dM, dsh, cb);
+            else
+              ok = chol_blk<T, 1, true>(p, S.Mb, ldM, S.dM, dsh, cb);
+            if (threadIdx.x == 0) *pd = ok ? 1 : 0;
+          }
+          cluster_barrier(S.D.blocks);
+          return *pd != 0;
+        }
         if (nt <= NTHREADS) return chol_blk<T, 1, true>(p, S.Mb, ldM, S.dM, dsh, cb);
         if constexpr (sizeof(T) == 4) {
           if (reg_chol_ok(p, 4)) return chol_blk<T, 2, true>(p, S.Mb, ldM, S.dM, dsh, cb);

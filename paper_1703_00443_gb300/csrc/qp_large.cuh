@@ -116,9 +116,9 @@ __device__ __noinline__ bool gsweep_setup(int n, int nz, int p, int m, const T* 
     }
     __syncthreads();
     if (flag[0]) return false;   // the same pivots in every block, so all blocks return
-    // Phase B: replay the sweeps on every panel row.  Every block forms the whole panels from
-    // the matrix; with several blocks the rows' new values are written by their owners once
-    // all blocks have read the old ones.
+    // Phase B: replay the sweeps on every panel row.  Panels in shared memory: every block forms them
+    // whole from the matrix, and with several blocks the rows' new values are written by their owners
+    // once all blocks have read the old ones.  In global memory the owners write the panels' rows too.
     auto replay = [&](int i, bool panels, bool write) {
       T* row = SR + (size_t)i * ldS + k0;
       T v[LNB];
@@ -150,8 +150,8 @@ __device__ __noinline__ bool gsweep_setup(int n, int nz, int p, int m, const T* 
       }
     };
     for (int pass = 0; pass < (blocks > 1 ? 2 : 1); ++pass) {
-      const int step = pass == 0 ? NTHREADS : gthreads;
-      for (int i = pass == 0 ? tid : gtid; i < N; i += step)
+      const bool whole = pass == 0 && pan_in_sm;
+      for (int i = whole ? tid : gtid; i < N; i += whole ? NTHREADS : gthreads)
         if (i < k0 || i >= k0 + LNB) replay(i, pass == 0, pass == 1 || blocks == 1);
       if (pass == 0) cluster_barrier(blocks);
     }

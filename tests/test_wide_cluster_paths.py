@@ -46,3 +46,21 @@ def test_equality_constrained(n, m):
     assert rel_err(outs[0][2].double().numpy()[None], [sols[0]["z"]]).max() <= 1e-5
     assert rel_err(outs[0][6].double().numpy()[None], [refs[0]["dq"]],
                    1e-3 * np.linalg.norm(g, axis=1)).max() <= 1e-4
+
+
+@pytest.mark.parametrize("n,p,m,dtype", [
+    (352, 120, 4, np.float32),       # register-tile Cholesky, one slot a thread
+    (356, 170, 9, np.float32),       # two slots
+    (480, 160, 40, np.float64),      # blocked Cholesky and sweep in FP64, the sweep's panels in global memory
+    (352, 40, 4, np.float64),        # register-tile Cholesky in FP64
+])
+def test_factorisations(n, p, m, dtype):
+    batch, g = _plain(n, p, m, dtype)
+    data = [x[0] for x in (batch.Q, batch.q, batch.G, batch.h, batch.A, batch.b)]
+    outs = [_run(data, g[0], B) for B in BATCHES]
+    assert int(outs[0][0]) == 0 and all(_same(outs[0], o) for o in outs[1:])
+    sols, refs = oracle_solve_and_grad(batch, g, [0])
+    ztol, gtol = (1e-5, 1e-4) if dtype == np.float32 else (1e-9, 1e-8)
+    assert rel_err(outs[0][2].double().numpy()[None], [sols[0]["z"]]).max() <= ztol
+    assert rel_err(outs[0][6].double().numpy()[None], [refs[0]["dq"]],
+                   1e-3 * np.linalg.norm(g, axis=1)).max() <= gtol
