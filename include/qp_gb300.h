@@ -114,6 +114,11 @@ int qp_supported(int dtype, int n, int nineq, int neq);
  * workspace, L2-resident), 0 if on the shared-memory kernel, −1 on invalid arguments. */
 int qp_uses_global_path(int dtype, int n, int nineq, int neq);
 
+/* Host query: thread blocks that share each instance of a qp_forward batch of B on the current device
+ * (1, 2, 4 or 8; large instances of small batches run on several SMs), −1 on invalid arguments.
+ * The results do not depend on it. */
+int qp_blocks_per_instance(const qp_options* opt, int dtype, int B, int n, int nineq, int neq);
+
 /* 1 if qp_forward's setup factorisation of this size (§3.1: the blocks of the KKT matrix that
  * do not change over the iterations, factored once) runs its rank-64 updates on the tensor
  * cores (tcgen05, TF32 with a three-term split that keeps FP32 accuracy): FP32 instances on

@@ -118,6 +118,7 @@ EXPORTS = {
     "qp_workspace_bytes_opt": (c_size_t, [ctypes.POINTER(QPOptions), c_int, c_int, c_int, c_int, c_int]),
     "qp_supported": (c_int, [c_int, c_int, c_int, c_int]),
     "qp_uses_global_path": (c_int, [c_int, c_int, c_int, c_int]),
+    "qp_blocks_per_instance": (c_int, [ctypes.POINTER(QPOptions)] + [c_int] * 5),
     "qp_uses_tensor_cores": (c_int, [ctypes.POINTER(QPOptions), c_int, c_int, c_int, c_int]),
     "qp_forward": (c_int, [ctypes.POINTER(QPOptions), c_int, c_int, c_int, c_int, c_int]
                    + [c_void_p] * 13 + [c_size_t, c_void_p]),

@@ -228,9 +228,6 @@ double est_cost(int n, int nz, int p, int m, bool large) {
 // fragmentation.  One n = 500 instance, forward and backward: 25.9 ms on one block of the
 // one-block kernels, 12.9 ms on eight; what is left is the chains that every block waits for.
 int blocks_per_instance(int B, bool share) {
-#if defined(QP_HOST_EMULATION)
-  return 1;   // the host emulation runs one block at a time
-#endif
   const int nsm = num_sms();
   if (!share) return 1;
   if (B * 8 <= nsm * 3 / 4) return 8;
@@ -357,6 +354,13 @@ int qp_supported(int dtype, int n, int nineq, int neq) {
 int qp_uses_global_path(int dtype, int n, int nineq, int neq) {
   if ((dtype != QP_F32 && dtype != QP_F64) || !dims_ok(1, n, nineq, neq)) return -1;
   return make_plan(dtype, n, nineq, neq).large ? 1 : 0;
+}
+
+int qp_blocks_per_instance(const qp_options* opt, int dtype, int B, int n, int nineq, int neq) {
+  if ((dtype != QP_F32 && dtype != QP_F64) || !dims_ok(B, n, nineq, neq)) return -1;
+  const Plan pl = make_plan(dtype, n, nineq, neq, opt ? opt->path : 0);
+  if (!pl.ok) return -1;
+  return blocks_per_instance(B, pl.share);
 }
 
 int qp_uses_tensor_cores(const qp_options* opt, int dtype, int n, int nineq, int neq) {
@@ -614,11 +618,7 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
   int np = 0;
   const int nwide = std::min(std::max(sizes->reserved >> 8, 0), ng);
   const int nshare = std::min(sizes->reserved & 255, nwide);
-#if defined(QP_HOST_EMULATION)
-  const Levels lv{0, 0, 0};   // the host emulation runs one block at a time
-#else
   const Levels lv = share_levels(nshare, share_sms(sizes, nsm));
-#endif
   int off = 0;
   auto add = [&](int kind, int cnt) {
     if (cnt > 0) parts[np++] = {kind, off, cnt};

@@ -21,11 +21,14 @@ cudaError_t launch_fwd_v(const FwdParams<T>& P, size_t smem, cudaStream_t st) {
 }
 template cudaError_t launch_fwd_v<QP_T, QP_SW, QP_CH>(const FwdParams<QP_T>&, size_t, cudaStream_t);
 #elif QP_KIND == 1
-#if !defined(QP_HOST_EMULATION)
 // A launch of clusters of `blocks` blocks, `count` of them.
 template <typename K, typename P>
 static cudaError_t launch_clusters(K kernel, const P& params, int count, int blocks, size_t smem,
                                    cudaStream_t st) {
+#if defined(QP_HOST_EMULATION)
+  emu_launch_clusters(kernel, count, blocks, smem, params);
+  return cudaSuccess;
+#else
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3((unsigned)(count * blocks));
   c.blockDim = dim3(NTHREADS);
@@ -38,17 +41,15 @@ static cudaError_t launch_clusters(K kernel, const P& params, int count, int blo
   c.attrs = &a;
   c.numAttrs = 1;
   return cudaLaunchKernelEx(&c, kernel, params);
-}
 #endif
+}
 template <typename T>
 cudaError_t launch_fwd_large_v(const FwdParams<T>& P, size_t smem, cudaStream_t st) {
   auto k = P.blocks == 0 ? qp_fwd_large_kernel<T, 0>
                          : (P.blocks == 1 ? qp_fwd_large_kernel<T, 1> : qp_fwd_large_kernel<T, 2>);
   cudaError_t e = prepare_smem(k, smem);
   if (e != cudaSuccess) return e;
-#if !defined(QP_HOST_EMULATION)
   if (P.blocks > 1) return launch_clusters(k, P, P.B, P.blocks, smem, st);
-#endif
   k<<<P.B, NTHREADS, smem, st>>>(P);
   return cudaGetLastError();
 }
@@ -59,9 +60,7 @@ cudaError_t launch_fwd_packed_large_v(const PackedFwdParams<T>& P, size_t smem, 
                          : (P.blocks == 1 ? qp_fwd_packed_large_kernel<T, 1> : qp_fwd_packed_large_kernel<T, 2>);
   cudaError_t e = prepare_smem(k, smem);
   if (e != cudaSuccess) return e;
-#if !defined(QP_HOST_EMULATION)
   if (P.blocks > 1) return launch_clusters(k, P, P.B, P.blocks, smem, st);
-#endif
   k<<<P.B, NTHREADS, smem, st>>>(P);
   return cudaGetLastError();
 }

@@ -1,6 +1,7 @@
 // Runs qp_forward + qp_backward_ext of the C ABI, compiled for the host with the emulation
 // shims, on one input file, and writes the results.
 // Input: int32 B, n, nineq, neq, dtype, path; then Q, q, G, h, A, b, dl_dz of the dtype.
+// EMU_MAX_ITER and EMU_TIME_LIMIT_US set those options.
 // Output: z, lam, nu, dQ, dq, dG, dh, dA, db, then int32 status[B], backward status[B].
 #include <cstdio>
 #include <cstdlib>
@@ -10,8 +11,8 @@
 #include "shim.h"
 
 thread_local EmuDim3 threadIdx, blockIdx;
-unsigned char* emu_dyn_smem = nullptr;
-EmuBlock* emu_blk = nullptr;
+thread_local unsigned char* emu_dyn_smem = nullptr;
+thread_local EmuBlock* emu_blk = nullptr;
 
 static void* xalloc(size_t bytes, int fill) {
   void* p = nullptr;
@@ -42,6 +43,8 @@ int main(int argc, char** argv) {
   qp_options o;
   qp_default_options(dtype, &o);
   o.path = hdr[5];
+  if (const char* v = getenv("EMU_MAX_ITER")) o.max_iter = atoi(v);
+  if (const char* v = getenv("EMU_TIME_LIMIT_US")) o.time_limit_us = atoi(v);
   const size_t wsb = qp_workspace_bytes_opt(&o, dtype, B, n, p, m);
   void* ws = xalloc(wsb, 0xff);   // as uninitialised as device memory may be
   void* z = xalloc((size_t)B * n * es, 0);

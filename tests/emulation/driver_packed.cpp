@@ -12,8 +12,8 @@
 #include "shim.h"
 
 thread_local EmuDim3 threadIdx, blockIdx;
-unsigned char* emu_dyn_smem = nullptr;
-EmuBlock* emu_blk = nullptr;
+thread_local unsigned char* emu_dyn_smem = nullptr;
+thread_local EmuBlock* emu_blk = nullptr;
 
 static void* xalloc(size_t bytes, int fill) {
   void* p = nullptr;

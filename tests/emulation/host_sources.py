@@ -28,7 +28,11 @@ def generate(out):
         dev = dev.replace(a, b)
     if "asm" in re.sub(r"//.*", "", dev):
         raise RuntimeError("inline assembly without a host equivalent")
-    dev = re.sub(r"\b__shared__\b", "static", dev)   # one block at a time: statics are per block
+    # static shared memory: one object for each of up to 16 blocks side by side
+    dev = re.sub(r"__shared__ ([\w ]+(?:<T>)?) (\w+);",
+                 r"static \1 \2_of[16]; auto& \2 = \2_of[blockIdx.x % 16];", dev)
+    if "__shared__" in re.sub(r"//.*", "", dev):
+        raise RuntimeError("shared memory without a host equivalent")
     dev = dev.replace("__stcs(", "emu_stcs(")
     open(os.path.join(out, "qp_device.cuh"), "w").write(dev)
     # the tensor-core routines are device-only (under __CUDA_ARCH__); the host build takes
@@ -38,6 +42,7 @@ def generate(out):
     if "asm" in re.sub(r"//.*", "", tc):
         raise RuntimeError("inline assembly left in qp_tc.cuh")
     # the wrappers' host definitions come before the routine that uses them
+    tc = tc.replace("  __syncthreads();   // a cluster of one", "  emu_cluster_barrier();")
     tc = tc.replace("// Bounded wait for the completion", '}  // namespace qpk\n#include "tc_emu.h"\n'
                     "namespace qpk {\n// Bounded wait for the completion", 1)
     open(os.path.join(out, "qp_tc.cuh"), "w").write(tc)

@@ -1,5 +1,5 @@
 // Host stand-ins for the CUDA runtime calls the library's host code makes, and the launch of
-// a kernel as blocks of host threads (one block after another).
+// a kernel as blocks of host threads (one cluster after another).
 #pragma once
 #include "shim.h"
 typedef int cudaError_t;
@@ -12,7 +12,8 @@ enum cudaFuncAttribute { cudaFuncAttributeMaxDynamicSharedMemorySize = 8 };
 #define cudaEventDisableTiming 2u
 inline cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 inline cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
-  *v = a == cudaDevAttrMultiProcessorCount ? 152 : 232448;   // GB300
+  const char* sms = getenv("EMU_SMS");   // another number of SMs than GB300's, for clusters of few blocks
+  *v = a == cudaDevAttrMultiProcessorCount ? (sms ? atoi(sms) : 152) : 232448;
   return cudaSuccess;
 }
 inline cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
@@ -29,27 +30,37 @@ inline cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = (vo
 // Shared memory is filled with 0xff bytes (NaN in either float type), so a read before the
 // kernel writes shows up in the results.
 template <class P>
-void emu_launch(void (*kernel)(const P), int grid, size_t smem, const P& params) {
+void emu_launch_clusters(void (*kernel)(const P), int count, int blocks, size_t smem, const P& params) {
   constexpr int kThreads = 512;
-  for (int b = 0; b < grid; ++b) {
-    EmuBlock blk;
-    blk.block = std::make_unique<std::barrier<>>(kThreads);
-    for (int w = 0; w < 32; ++w) blk.warp[w] = std::make_unique<std::barrier<>>(32);
-    emu_blk = &blk;
-    void* s = nullptr;
-    if (posix_memalign(&s, 128, smem ? smem : 16) != 0) abort();
-    std::memset(s, 0xff, smem ? smem : 16);
-    emu_dyn_smem = (unsigned char*)s;
+  for (int c = 0; c < count; ++c) {
+    std::barrier<> cluster(kThreads * blocks);
+    std::vector<EmuBlock> blk(blocks);
+    std::vector<void*> dyn(blocks);
+    for (int r = 0; r < blocks; ++r) {
+      blk[r].cluster = &cluster;
+      blk[r].block = std::make_unique<std::barrier<>>(kThreads);
+      for (int w = 0; w < 32; ++w) blk[r].warp[w] = std::make_unique<std::barrier<>>(32);
+      if (posix_memalign(&dyn[r], 128, smem ? smem : 16) != 0) abort();
+      std::memset(dyn[r], 0xff, smem ? smem : 16);
+    }
     std::vector<std::thread> th;
-    for (int t = 0; t < kThreads; ++t)
-      th.emplace_back([&, t, b] {
-        threadIdx.x = t;
-        blockIdx.x = b;
-        kernel(params);
-        emu_blk->warp[t >> 5]->arrive_and_drop();
-        emu_blk->block->arrive_and_drop();
-      });
+    for (int r = 0; r < blocks; ++r)
+      for (int t = 0; t < kThreads; ++t)
+        th.emplace_back([&, r, t, c] {
+          emu_blk = &blk[r];
+          emu_dyn_smem = (unsigned char*)dyn[r];
+          threadIdx.x = t;
+          blockIdx.x = c * blocks + r;
+          kernel(params);
+          emu_blk->warp[t >> 5]->arrive_and_drop();
+          emu_blk->block->arrive_and_drop();
+          cluster.arrive_and_drop();
+        });
     for (auto& x : th) x.join();
-    free(s);
+    for (void* p : dyn) free(p);
   }
+}
+template <class P>
+void emu_launch(void (*kernel)(const P), int grid, size_t smem, const P& params) {
+  emu_launch_clusters(kernel, grid, 1, smem, params);
 }

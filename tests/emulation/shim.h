@@ -1,6 +1,7 @@
 // Host emulation of the CUDA device features the library's kernels use, for CPU checks of
-// the kernel source: one thread block runs as NTHREADS std::threads, __syncthreads and
-// __syncwarp are std::barrier waits, and warp shuffles go through a per-warp exchange
+// the kernel source: a thread block runs as NTHREADS std::threads (the blocks of a cluster side by
+// side, other blocks one after another), __syncthreads, __syncwarp and the cluster barrier
+// are std::barrier waits, and warp shuffles go through a per-warp exchange
 // buffer between two warp barriers (so a shuffle that not every lane of a warp reaches
 // deadlocks here, as it may hang a GPU).  Shared memory is a heap buffer of the launch's
 // exact size, so AddressSanitizer sees any access past it.
@@ -38,16 +39,18 @@ inline double2 make_double2(double a, double b) { return {a, b}; }
 
 struct EmuDim3 { unsigned x = 0, y = 0, z = 0; };
 extern thread_local EmuDim3 threadIdx, blockIdx;
-extern unsigned char* emu_dyn_smem;
+extern thread_local unsigned char* emu_dyn_smem;
 
 struct EmuBlock {
+  std::barrier<>* cluster = nullptr;
   std::unique_ptr<std::barrier<>> block;
   std::unique_ptr<std::barrier<>> warp[32];
   alignas(16) unsigned char xbuf[32][32][8];
 };
-extern EmuBlock* emu_blk;
+extern thread_local EmuBlock* emu_blk;
 
 inline void __syncthreads() { emu_blk->block->arrive_and_wait(); }
+inline void emu_cluster_barrier() { emu_blk->cluster->arrive_and_wait(); }
 inline void __syncwarp(unsigned = 0xffffffffu) { emu_blk->warp[threadIdx.x >> 5]->arrive_and_wait(); }
 
 template <class T>

@@ -1,6 +1,5 @@
 // Host emulation of the tensor-core, bulk-copy and mbarrier wrappers of qp_tc.cuh, for the
-// CPU check of the kernel source.  Blocks run one at a time, so one tensor-memory array
-// serves every block.  MMAs complete when issued; an mbarrier word holds the number of
+// CPU check of the kernel source.  MMAs complete when issued; an mbarrier word holds the number of
 // completed phases.
 // The operand layouts are read exactly as the descriptors describe them (start address,
 // leading- and stride-dimension byte offsets of the canonical K-major layout), so a layout
@@ -20,8 +19,8 @@ struct EmuTmem {
   int cols = 0;
 };
 inline EmuTmem& emu_tmem() {
-  static EmuTmem* t = new EmuTmem();
-  return *t;
+  static EmuTmem* t = new EmuTmem[16];   // of the blocks side by side
+  return t[blockIdx.x % 16];
 }
 [[noreturn]] inline void emu_tc_fail(const char* what) {
   fprintf(stderr, "tensor-core emulation: %s\n", what);
@@ -94,7 +93,16 @@ inline void tc_mma_tf32(uint32_t tmem, const void* a, const void* b, uint32_t lb
       t.v[i][col0 + j] = s;
     }
 }
-inline void tc_commit(uint64_t* bar) { emu_bar_complete(bar); }
+// EMU_LATE_BLOCK: that block's third commit never arrives, so its waits on it run out.
+inline int emu_late_block() {
+  static const int b = getenv("EMU_LATE_BLOCK") ? atoi(getenv("EMU_LATE_BLOCK")) : -1;
+  return b;
+}
+inline void tc_commit(uint64_t* bar) {
+  static std::atomic<int> commits{0};
+  if (emu_late_block() == (int)blockIdx.x && commits.fetch_add(1) == 2) return;
+  emu_bar_complete(bar);
+}
 inline void tc_ld32(uint32_t taddr, float (&v)[32]) {
   EmuTmem& t = emu_tmem();
   const int lane0 = (int)(taddr >> 16), col = (int)(taddr & 0xFFFF);
@@ -106,12 +114,13 @@ inline void tc_ld32(uint32_t taddr, float (&v)[32]) {
 inline void tc_fence_before() { __atomic_thread_fence(__ATOMIC_SEQ_CST); }
 inline void tc_fence_after() { __atomic_thread_fence(__ATOMIC_SEQ_CST); }
 inline void tc_proxy_fence() { __atomic_thread_fence(__ATOMIC_SEQ_CST); }
-// A virtual clock for the bounded waits: 1 µs per reading, so a wait gives up after about
+// A virtual clock for the bounded waits, one per block: 1 µs per reading, so a wait gives up after about
 // 32 million polls whatever the host's load (a barrier that never completes still ends the
-// wait, as on the GPU).
+// wait, as on the GPU); 20 µs in a block whose wait is to run out.
 inline unsigned long long tc_now() {
-  static std::atomic<unsigned long long> t{0};
-  return t.fetch_add(1000, std::memory_order_relaxed);
+  static std::atomic<unsigned long long> t[16];
+  return t[blockIdx.x % 16].fetch_add(emu_late_block() == (int)blockIdx.x ? 20000 : 1000,
+                                      std::memory_order_relaxed);
 }
 
 }  // namespace qpk
