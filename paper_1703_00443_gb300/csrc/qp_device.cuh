@@ -2538,7 +2538,7 @@ __device__ __forceinline__ void init_global_path(GlobalPath<T>& S, const FwdInst
   S.tcp = TC && S.L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr;
   // exchange buffer of the cluster's blocks: the panel scratch, idle outside the factorisations
   // (and in them where the panels are in shared memory)
-  S.D = Dist<T>{blocks, rank, S.pan, (int)((W.oTc - W.oPan) / sizeof(T)), S.L.ring ? sm + S.L.ocb : nullptr,
+  S.D = Dist<T>{S.L.pan_smem ? blocks : 1, rank, S.pan, (int)((W.oTc - W.oPan) / sizeof(T)), S.L.ring ? sm + S.L.ocb : nullptr,
                 S.L.ring ? (int)(S.L.cbytes - RING_BYTES) : 0};
 }
 template <typename T, bool TC, int WIDE>
@@ -2601,6 +2601,11 @@ __device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned ch
     __shared__ GlobalPath<T> S;
     if (threadIdx.x == 0) init_global_path<T, TC>(S, I, sm, blocks, rank);
     __syncthreads();
+    // Panels in global memory are where the blocks would exchange: one block then, whatever the plan says
+    // (the planner shares no such instance, but a plan may come from anywhere).
+    if constexpr (WIDE == 2) {
+      if (!S.L.pan_smem && rank > 0) return;
+    }
     run_global_path<T, TC, WIDE>(S, sm);
   } else {
     GlobalPath<T> S;

@@ -141,3 +141,20 @@ def test_a_streams_first_packed_call_may_be_captured():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out.z, ref)
+
+
+def test_a_plan_that_shares_what_cannot_be_shared():
+    """`reserved` of another origin: 700 inequalities have their panels in global memory, where the
+    blocks of a cluster would exchange.  One block takes the instance; a size below the wide line runs
+    on a cluster as well."""
+    for size in ((700, 700, 0), (200, 200, 50)):
+        t = tuple(np.float32(x) for x in inputs.random_qp(*size, workload=inputs.WL_UNEVEN, index=3))
+        z = []
+        for reserved in (1 << 8, 1 << 8 | 1):
+            pb = PackedBatch([size], device=DEV)
+            pb.sizes.reserved = reserved
+            out = pb.forward(*pb.pack([t]))
+            torch.cuda.synchronize()
+            assert int(out.status[0]) == 0
+            z.append(out.z.clone())
+        assert torch.equal(*z), size
