@@ -225,8 +225,10 @@ double est_cost(int n, int nz, int p, int m, bool large) {
 // batch's clusters are resident at once (one block per SM; a cluster needs its SMs within one
 // processing cluster of 16 to 20, which leaves a few SMs unused), one block otherwise.  The
 // shares taken of the SMs (3/4 for clusters of eight, 9/10 for the others) are that
-// fragmentation.  One n = 500 instance, forward and backward: 25.9 ms on one block of the
-// one-block kernels, 12.9 ms on eight; what is left is the chains that every block waits for.
+// fragmentation.  One n = 500 instance, forward and backward: 25.5 ms on one block of the
+// other sizes' kernel, 11.7 ms on eight; what is left is the chains that every block waits for.
+// (The batch is taken to have the device to itself: several calls in flight on streams of
+// their own, each of a few large instances, get more out of one packed batch.)
 int blocks_per_instance(int B, bool share) {
   const int nsm = num_sms();
   if (!share) return 1;
@@ -238,9 +240,10 @@ int blocks_per_instance(int B, bool share) {
 
 // Blocks of the leading `nshare` wide instances of a packed batch, largest first: all of them
 // resident at once, so two blocks each, then four for as many as the SMs hold, then eight.
-// Clusters that wait for their turn cost more than they give (256 mixed requests, 46 shared: at
-// four blocks each 21.1 ms, at four and two all resident 17.6), and blocks left idle are worth
-// most to the largest (96 requests, 24 shared: at four 15.4 ms, the first ten at eight 13.0).
+// Clusters that wait for their turn cost more than they give (256 mixed requests, 46 shared, by an
+// earlier form of the kernels: at four blocks each 21.1 ms, at four and two all resident 17.6), and
+// blocks left idle are worth most to the largest (96 requests, 24 shared: at four 15.4 ms, the
+// first ten at eight 13.0).  So eight and two never meet in one batch.
 struct Levels { int n8, n4, n2; };   // instances at eight, four and two blocks, in this order
 int share_most(int nsm) { return nsm * 9 / 10 / 2; }   // instances that have room for two blocks each
 Levels share_levels(int nshare, int nsm) {
@@ -388,7 +391,10 @@ int qp_forward(const qp_options* opt, int dtype, int B, int n, int nineq, int ne
   if (workspace_bytes < (size_t)B * pl.ws) return QP_ENOSPACE;
   if (!pl.ok) return QP_EUNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
-  const int blocks = pl.wide ? blocks_per_instance(B, pl.share) : 0;
+  // (Without inequalities a wide size has no dealt products: on one block it runs on the kernel of the
+  // other sizes, the same arithmetic; n = 352, batch 128 1.19 ms against 1.22.)
+  int blocks = pl.wide ? blocks_per_instance(B, pl.share) : 0;
+  if (blocks == 1 && nineq == 0) blocks = 0;
   cudaError_t e;
   if (dtype == QP_F32) {
     qpk::FwdParams<float> P{B, n, nineq, neq, pl.nz,
@@ -607,8 +613,8 @@ int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance
                 : qpk::launch_fwd_packed_f64(P, sizes->sw, sizes->ch & 255, (size_t)sizes->fwd_smem,
                                              grid, s);
   };
-  // Up to six kernels side by side: the largest wide instances with eight, four and two blocks
-  // each (first in the descriptor array), the other wide ones, the other global-path ones, and the
+  // Up to five kernels side by side: the largest wide instances with eight and four or four and two
+  // blocks each (first in the descriptor array), the other wide ones, the other global-path ones, and the
   // shared-memory-path ones; the first of them on `stream`, the others on side streams forked
   // from it and joined back to it, launched in this order so that the costliest take the SMs
   // first.  A block holds its SM until it ends (the last kernel's until its queue runs dry), so
