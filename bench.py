@@ -494,7 +494,7 @@ def run_gpu(args):
             e2e_ms.append(e0.elapsed_time(e1))
     clocks = sampler.stop()
 
-    # The same 128 instances through the packed (persistent, uneven-capable) path.
+    # The same 128 instances through the packed (uneven-capable) path.
     packed_ms = None
     if not args.no_extras:
         from paper_1703_00443_gb300.packed import PackedBatch
@@ -582,7 +582,7 @@ def run_gpu(args):
         "gpu_launches": 2 * args.steps,
         "batched_vs_plain": None if packed_ms is None else {
             "plain_fixed_size_ms_per_step": step_ms, "packed_persistent_ms_per_step": packed_ms,
-            "note": "same 128 instances; packed = one persistent launch per direction over descriptors"},
+            "note": "same 128 instances; packed = kernels over descriptors of the instances"},
         "uneven": uneven,
         "served": served,
         "clocks": clocks,
@@ -620,8 +620,8 @@ def _time_fixed(Tin, gdev, steps, flush, stream):
 
 def uneven_run(dev, count, steps, tuned, flush, stream):
     """The uneven workload: `count` QPs with n ~ U{8..256}, nineq ~ U{n/2..2n}, neq ~ U{0..n/4}
-    as one packed batch, forward (global-path and shared-memory-path instances in two
-    persistent kernels side by side) + backward (one persistent kernel), L2 flushed between
+    as one packed batch, forward (global-path instances one block each, shared-memory-path
+    ones in a persistent kernel beside them) + backward (one persistent kernel), L2 flushed between
     steps.  tuned: the autotuner's path choice and cost model."""
     import torch
     from paper_1703_00443_gb300 import inputs
@@ -712,7 +712,7 @@ def run_workload(args):
                                 args.serve_count, args.serve_inflight, _classes(args),
                                 args.serve_max_batch))
     elif args.workload == "uneven":
-        line.update({"metric": "uneven batch fwd+bwd solves/sec (two persistent kernels forward, one backward)"})
+        line.update({"metric": "uneven batch fwd+bwd solves/sec (kernels side by side forward, one persistent backward)"})
         line.update(uneven_run(dev, args.uneven_count, args.uneven_steps, args.tuned, flush, stream))
     print(json.dumps(line), flush=True)
 

@@ -263,11 +263,11 @@ int qp_packed_blocks(const qp_packed_sizes* sizes, int32_t* counts);
 
 /* Forward pass of a packed batch (device pointers as in qp_forward, packed as above;
  * status/iters/resid indexed by instance id; workspace of sizes->ws_bytes bytes).  The
- * instances shared by eight, four and two blocks, the other wide ones, the other global-path ones and the
- * shared-memory-path ones run as up to six kernels side by side: the first on `stream`, the
+ * instances shared by eight and four or by four and two blocks, the other wide ones, the other
+ * global-path ones and the shared-memory-path ones run as up to five kernels side by side: the first on `stream`, the
  * others on library-owned side streams forked from `stream` and joined back to it by events
- * (one set per caller stream, for up to 16 streams per device; created on a stream's first
- * such call: make that call before any stream capture).  Later kernels' blocks take SMs as
+ * (one set per caller stream, for up to 16 streams per device, as many as its calls need;
+ * created with the call, also under stream capture).  Later kernels' blocks take SMs as
  * the earlier ones' blocks end. */
 int qp_forward_packed(const qp_options* opt, int dtype, int B, const qp_instance_desc* desc,
                       const qp_packed_sizes* sizes, const void* Q, const void* q,

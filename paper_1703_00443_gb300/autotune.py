@@ -1,12 +1,12 @@
 """Measured tuning of the packed-batch schedule: which kernel path each size takes and the
-cost model that orders the persistent work queue.
+cost model that orders the instances.
 
 ``measure`` times one wave of instances (one block per SM, so the time is one instance's
 latency) for a grid of size classes on every kernel path that can take them; ``fit`` fits,
 per path, time ≈ c·[sweep FMAs, per-iteration Schur FMAs, residual FMAs, 1] by least squares;
 ``Tuning.plan_arrays`` then picks, for each instance of a packed batch, the path with the
 smaller predicted time (where both are possible) and hands the predicted times to the
-planner, which orders the work queue largest first.  ``autotune`` runs all three and saves
+planner, which orders the instances largest first.  ``autotune`` runs all three and saves
 the table as JSON (by default next to the built library).
 """
 from __future__ import annotations

@@ -2694,8 +2694,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_kernel(const Packed
 // estimated cost first), which the block scheduler follows: no work queue, and no second
 // path's code and spills in the kernel.  Bound by the longest instance's chain, then by the L2
 // traffic of the factors of 152 instances in flight.  512 uneven instances, forward and
-// backward: 17.4 ms with a persistent kernel of both paths, 16.9 ms now.  The setup sweep runs on CUDA cores (its tensor-core form faulted
-// in an earlier persistent form of this kernel, for a reason that was not found).
+// backward: 17.8 ms with a persistent kernel of both paths, 17.0 ms now (most of it since the
+// tensor-core routine, never called here, is not compiled in).  The setup sweep runs on CUDA cores
+// (its tensor-core form faulted in an earlier persistent form of this kernel, for a reason that was
+// not found).
 template <typename T, int WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1) qp_fwd_packed_large_kernel(const PackedFwdParams<T> P) {
   extern __shared__ __align__(16) unsigned char sm[];

@@ -1,6 +1,6 @@
 """Packed batches of QPs of uneven sizes (C ABI ``qp_packed_plan`` / ``qp_forward_packed`` /
 ``qp_backward_packed``): each instance on the kernel path its own size selects, largest
-estimated cost first; up to six kernels side by side forward, one backward.
+estimated cost first; up to five kernels side by side forward, one backward.
 
     pb = PackedBatch([(n0, nineq0, neq0), (n1, nineq1, neq1), ...])
     Qp, qp, Gp, hp, Ap, bp = pb.pack(instances)        # flat device tensors
