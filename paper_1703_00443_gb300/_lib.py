@@ -28,6 +28,7 @@ def _variants():
     out = []
     for T, tag, pairs in (("float", "f32", [(1, 1), (2, 1), (4, 1), (4, 2)]),
                           ("double", "f64", [(1, 1), (2, 1)])):
+        out.append((f"fwd_{tag}_wide", "qp_fwd_variant", [f"-DQP_T={T}", "-DQP_KIND=3"]))
         out.append((f"fwd_{tag}_large", "qp_fwd_variant", [f"-DQP_T={T}", "-DQP_KIND=1"]))
         for kind, kname in ((0, "plain"), (2, "packed")):
             for sw, ch in pairs:

@@ -171,7 +171,9 @@ struct FwdSmem {
   size_t oSR, oMb, odM, ocb, cbytes, odbl, osplit, ovec, ored, total;
   // large: S/RE, M/X and diag(M) live in the global workspace, only vectors and a work
   // region stay in shared memory.
-  __host__ __device__ void init(int n, int nzp, int p, int m, bool large) {
+  // may_ring = false: without the room for the dealt products' copies (the kernel of the sizes below the
+  // wide line; a layout without it is never larger).
+  __host__ __device__ void init(int n, int nzp, int p, int m, bool large, bool may_ring = true) {
     nz = nzp;
     m1 = nz + m;
     N3 = m1 + p;
@@ -233,7 +235,7 @@ struct FwdSmem {
         if (TC_SMEM_BYTES > cbytes) cbytes = align_up(TC_SMEM_BYTES, 16);
       }
       // Room for the dealt products' copies, if it fits.
-      ring = wide_size(m1) && o + (cbytes > RING_BYTES ? cbytes : RING_BYTES) + tail <= LARGE_PANEL_SMEM_CAP;
+      ring = may_ring && wide_size(m1) && o + (cbytes > RING_BYTES ? cbytes : RING_BYTES) + tail <= LARGE_PANEL_SMEM_CAP;
       if (ring && RING_BYTES > cbytes) cbytes = RING_BYTES;
     }
     o += cbytes;
@@ -2518,7 +2520,7 @@ __device__ __forceinline__ void fwd_smem_path(const FwdInst<T>& I, unsigned char
 // persistent one raised a GPU fault whose cause was not found), so their workspaces have no
 // panel-tile region.
 template <typename T>
-struct GlobalPath {   // an instance, its layout and its matrices in the workspace
+struct GlobalPath {   // a wide instance, its layout and its matrices in the workspace (shared memory)
   FwdInst<T> I;
   FwdSmem<T> L;
   Dist<T> D;
@@ -2587,8 +2589,7 @@ __device__ __forceinline__ void run_global_path(const GlobalPath<T>& S, unsigned
       [&](const T* rhs, T* y, T* out, T* scr) {
         const int p = S.I.p, ldM = p > 0 ? p : 1;
         if (reg_chol_ok(p, (int)sizeof(T))) {
-          if constexpr (WIDE != 0) chol_solve_call(p, S.Mb, ldM, rhs, y, out, scr);
-          else chol_solve(p, S.Mb, ldM, rhs, y, out, scr);
+          chol_solve_call(p, S.Mb, ldM, rhs, y, out, scr);
         }
         else blk_solve(p, S.Mb, ldM, rhs, y, out, scr);
       },
@@ -2608,9 +2609,41 @@ __device__ __forceinline__ void fwd_global_path(const FwdInst<T>& I, unsigned ch
     }
     run_global_path<T, TC, WIDE>(S, sm);
   } else {
-    GlobalPath<T> S;
-    init_global_path<T, TC>(S, I, sm, 1, 0);
-    run_global_path<T, TC, 0>(S, sm);
+    // sizes below the wide line: everything in locals (as a GlobalPath object: n = 200, nineq = 150 1%
+    // slower, by the register allocation)
+    FwdSmem<T> L;
+    L.init(I.n, I.nz, I.p, I.m, true, false);
+    const int n = I.n, p = I.p, m = I.m, nz = I.nz;
+    WsLayout W;
+    W.init(n, nz, p, m, (int)sizeof(T), true, TC);
+    T* SR = reinterpret_cast<T*>(I.ws + W.oSR);
+    T* Mb = reinterpret_cast<T*>(I.ws + W.oX);
+    T* dM = reinterpret_cast<T*>(I.ws + W.odM);
+    T* Aw = reinterpret_cast<T*>(I.ws + W.oAw);
+    T* pan = reinterpret_cast<T*>(I.ws + W.oPan);
+    T* cb = reinterpret_cast<T*>(sm + L.ocb);
+    const Dist<T> D{1, 0, pan, (int)((W.oTc - W.oPan) / sizeof(T)), nullptr, 0};
+    fwd_body<T, true, 0>(I, L, sm, SR, Mb, p > 0 ? p : 1, dM, D,
+        [&](const T* Qb, const T* Ab, const T* Gb, T delta, T zthr) {
+          return gsweep_setup<T, false, TC>(n, nz, p, m, Qb, Ab, Gb, SR, Mb, dM, pan, L.span_smem != 0, cb,
+                                            delta, zthr,
+                                            TC && L.tc_sweep ? reinterpret_cast<T*>(I.ws + W.oTc) : nullptr,
+                                            1, 0);
+        },
+        [&](const T* dsh) {
+          const int NT = (p + 3) >> 2, nt = NT * (NT + 1) / 2, ldM = p > 0 ? p : 1;
+          if (nt <= NTHREADS) return chol_blk<T, 1, true>(p, Mb, ldM, dM, dsh, cb);
+          if constexpr (sizeof(T) == 4) {
+            if (reg_chol_ok(p, 4)) return chol_blk<T, 2, true>(p, Mb, ldM, dM, dsh, cb);
+          }
+          return gchol_factor<T, false>(p, Mb, dM, dsh, Aw, pan, L.pan_smem != 0, cb, pan, 1, 0);
+        },
+        [&](const T* rhs, T* y, T* out, T* scr) {
+          const int ldM = p > 0 ? p : 1;
+          if (reg_chol_ok(p, (int)sizeof(T))) chol_solve(p, Mb, ldM, rhs, y, out, scr);
+          else blk_solve(p, Mb, ldM, rhs, y, out, scr);
+        },
+        [](T*&, T*&, T*&) {});
   }
 }
 

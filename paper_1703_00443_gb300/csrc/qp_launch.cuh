@@ -26,6 +26,10 @@ cudaError_t launch_fwd_large_v(const FwdParams<T>& P, size_t smem, cudaStream_t 
 template <typename T, int SW, int CH>
 cudaError_t launch_fwd_packed_v(const PackedFwdParams<T>& P, size_t smem, int grid, cudaStream_t st);
 template <typename T>
+cudaError_t launch_fwd_wide_v(const FwdParams<T>& P, size_t smem, cudaStream_t st);
+template <typename T>
+cudaError_t launch_fwd_packed_wide_v(const PackedFwdParams<T>& P, size_t smem, cudaStream_t st);
+template <typename T>
 cudaError_t launch_fwd_packed_large_v(const PackedFwdParams<T>& P, size_t smem, cudaStream_t st);
 
 cudaError_t launch_fwd_f32(const FwdParams<float>& P, int SW, int CH, size_t smem, cudaStream_t st);

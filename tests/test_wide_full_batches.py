@@ -18,7 +18,7 @@ DEV = "cuda:0"
 def test_wide_kernels_hold_no_spilled_views_over_their_calls():
     """The wide kernels took 2656 bytes of spill loads in an iteration's body; that traffic goes to L2.
     A quarter of it is the bound (the compiler's own report, kept by the build)."""
-    log = os.path.join(_lib.BUILD, "fwd_f32_large.ptxas.log")
+    log = os.path.join(_lib.BUILD, "fwd_f32_wide.ptxas.log")
     if not os.path.exists(log):
         pytest.skip("the library was not built here")
     found = re.findall(r"Function properties for \S*qp_fwd_(?:packed_)?large_kernelIfL[ib]([12])E\S*\n"
@@ -28,10 +28,10 @@ def test_wide_kernels_hold_no_spilled_views_over_their_calls():
 
 def test_packed_kernels_carry_no_tensor_core_routine():
     """They never call it (by the compiler's report, kept by the build)."""
-    log = os.path.join(_lib.BUILD, "fwd_f32_large.ptxas.log")
-    if not os.path.exists(log):
+    logs = [os.path.join(_lib.BUILD, f"fwd_f32_{k}.ptxas.log") for k in ("large", "wide")]
+    if not all(os.path.exists(log) for log in logs):
         pytest.skip("the library was not built here")
-    kernels = open(log).read().split("Compiling entry function")[1:]
+    kernels = [k for log in logs for k in open(log).read().split("Compiling entry function")[1:]]
     packed = [k for k in kernels if "qp_fwd_packed_large_kernel" in k.split("\n")[0]]
     assert len(packed) == 3 and not any("tc_sweep_superblocks" in k for k in packed)
     assert sum("tc_sweep_superblocks" in k for k in kernels) == 3      # the fixed-size ones do
